@@ -141,12 +141,20 @@ struct Spectrum {
     double* g64 = nullptr;
     float* g32 = nullptr;
     dsf* gds = nullptr;
+    // the mixed spectrum (offset along the first axis, frequency along the
+    // other two) of the direct i pass; none for the finite box
+    double* m64 = nullptr;
+    float* m32 = nullptr;
+    dsf* mds = nullptr;
     double* near = nullptr;   // G_s on the offsets below NEAR_TN (preconditioner blocks)
     size_t bytes = 0;
     ~Spectrum() {
         if (g64) cudaFree(g64);
         if (g32) cudaFree(g32);
         if (gds) cudaFree(gds);
+        if (m64) cudaFree(m64);
+        if (m32) cudaFree(m32);
+        if (mds) cudaFree(mds);
         if (near) cudaFree(near);
     }
 };
@@ -255,7 +263,14 @@ struct SpectrumCache {
                 box_spectrum(N, s, 1.0 / (L * L * L), sp->g64, sp->g32, st);
                 to_dsf(sp->g64, n3, sp->gds, st);
             } else {
-                lgf_spectrum(N, s, 1.0 / (L * L * L), sp->g64, sp->g32, st);
+                const long long nm = (long long)N * (N + 1) * (N + 1);
+                alloc_check(nm * sizeof(double));
+                BAE_CUDA(cudaMalloc(&sp->m64, nm * sizeof(double)));
+                BAE_CUDA(cudaMalloc(&sp->m32, nm * sizeof(float)));
+                BAE_CUDA(cudaMalloc(&sp->mds, nm * sizeof(dsf)));
+                sp->bytes += nm * (sizeof(double) + sizeof(float) + sizeof(dsf));
+                lgf_spectrum(N, s, 1.0 / (L * L * L), sp->g64, sp->g32, st, 1.0 / (L * L), sp->m64, sp->m32);
+                to_dsf(sp->m64, nm, sp->mds, st);
                 to_dsf(sp->g64, n3, sp->gds, st);
                 alloc_check(NEAR_TAB * sizeof(double));
                 BAE_CUDA(cudaMalloc(&sp->near, NEAR_TAB * sizeof(double)));
@@ -366,6 +381,8 @@ bool problem_view(const bae_problem* P, ProblemView& out) {
     out.rec = P->geo.recipe();
     out.ghat64 = P->spec->g64;
     out.ghat32 = P->spec->g32;
+    out.gmix64 = P->spec->m64;
+    out.gmix32 = P->spec->m32;
     auto it = P->ctx->tw.find(2 * P->geo.N);
     if (it != P->ctx->tw.end()) {
         out.tw64 = it->second.tw64;
@@ -419,12 +436,15 @@ ConvArgs<T> conv_args(bae_problem* P, int nb, bool pruned = false) {
     const Twiddles& tw = P->ctx->twiddles(2 * N);
     if constexpr (std::is_same<T, dsf>::value) {
         a.ghat = P->spec->gds;
+        a.gmix = P->spec->mds;
         a.tw = tw.twds;
     } else if constexpr (sizeof(T) == 8) {
         a.ghat = reinterpret_cast<const T*>(P->spec->g64);
+        a.gmix = reinterpret_cast<const T*>(P->spec->m64);
         a.tw = reinterpret_cast<const cplx_t<T>*>(tw.tw64);
     } else {
         a.ghat = reinterpret_cast<const T*>(P->spec->g32);
+        a.gmix = reinterpret_cast<const T*>(P->spec->m32);
         a.tw = reinterpret_cast<const cplx_t<T>*>(tw.tw32);
     }
     return a;

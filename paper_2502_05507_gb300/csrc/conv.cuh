@@ -57,6 +57,10 @@ struct ConvArgs {
     cplx_t<T>* A = nullptr;
     cplx_t<T>* B = nullptr;
     const T* ghat = nullptr;      // (N+1)^3 octant, includes 1/(2N)^3
+    // the spectrum before its transform along the first axis (direct i pass):
+    // gmix[d][jj][kk], offset d < N, jj, kk <= N, includes 1/(2N)^2 (null:
+    // the i pass is always the FFT)
+    const T* gmix = nullptr;
     const cplx_t<T>* tw = nullptr;  // exp(-2 pi i m / 2N), m < 2N
     typename OutOf<T>::type* v = nullptr;   // [nbatch][N^3] output potential
     // x-planes [p0, p1) hold every nonzero source and every output the
@@ -102,6 +106,10 @@ template <typename T, int L>
 void run_conv(const ConvArgs<T>& a, cudaStream_t st);
 template <typename T, int L>
 void conv_configure();
+
+// The i pass as a direct sum (conv_direct_*.cu), in place in B.
+template <typename T>
+void launch_direct_i(const ConvArgs<T>& a, cudaStream_t st);
 
 // The cluster plane kernels (conv_cplane_*.cu) for L where one plane of
 // k-spectra does not fit one CTA: cplane_ready sets their attributes and

@@ -1,0 +1,8 @@
+// The direct i pass for float32.
+#include "conv_direct.cuh"
+
+namespace bae {
+
+template void launch_direct_i<float>(const ConvArgs<float>&, cudaStream_t);
+
+}  // namespace bae

@@ -161,8 +161,8 @@ __device__ __forceinline__ T source_value(const SrcRecipe& rec, int s, const dou
 // launch without the attribute makes the wait a no-op.
 __device__ __forceinline__ void wait_prior_grid() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
-template <typename K, typename A>
-void launch_pdl(K kernel, dim3 grid, int threads, size_t smem, cudaStream_t st, const A& a) {
+template <typename K, typename... A>
+void launch_pdl(K kernel, dim3 grid, int threads, size_t smem, cudaStream_t st, const A&... a) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
@@ -173,7 +173,7 @@ void launch_pdl(K kernel, dim3 grid, int threads, size_t smem, cudaStream_t st, 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    BAE_CUDA(cudaLaunchKernelEx(&cfg, kernel, a));
+    BAE_CUDA(cudaLaunchKernelEx(&cfg, kernel, a...));
 }
 
 // ------------------------------------------------ packed Nyquist column
@@ -285,5 +285,24 @@ template <typename T, int L> struct CPlaneGeo {
     static constexpr size_t SMEM = ROWS + (XL > XC ? XL : XC);
     static constexpr bool USE = CS > 1 && CS <= 8 && SMEM <= 227 * 1024 && NR % 2 == 0;
 };
+
+// Planes up to which the i pass is the direct sum (conv_direct.cuh): n^2
+// products per pencil against two transforms of length 2N, whatever n. The
+// lines lie where the two cross for one right-hand side (boundary operator of
+// spheres, microseconds with the direct sum / with the FFT i pass):
+//   float32:  N = 256 122 planes 383 / 459, 160 planes 605 / 540; N = 128 64
+//             planes 87 / 91, 82 planes 111 / 93; N <= 64 never (latency)
+//   double-float: N = 256 82 planes 909 / 1257, 122 planes 1557 / 1392;
+//             N = 128 64 planes 174 / 205, 82 planes 282 / 234; N = 64 44
+//             planes 86 / 86
+//   float64:  N = 256 122 planes 6887 / 8515; N = 128 82 planes 1057 / 1117,
+//             102 planes 1435 / 1231; N = 64 54 planes 214 / 229
+// (128 planes is also what the shared memory of the 8-byte types holds).
+template <typename T>
+inline int direct_i_limit(int N) {
+    if constexpr (std::is_same<T, float>::value) return N >= 256 ? 132 : (N >= 128 ? 68 : 0);
+    else if constexpr (std::is_same<T, dsf>::value) return N >= 256 ? 104 : (N >= 128 ? 70 : (N >= 64 ? 44 : 0));
+    else return N >= 256 ? 128 : (N >= 128 ? 84 : (N >= 64 ? 56 : 0));
+}
 
 }  // namespace bae

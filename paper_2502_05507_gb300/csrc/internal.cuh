@@ -16,6 +16,8 @@ struct ProblemView {
     SrcRecipe rec;
     const double* ghat64 = nullptr;   // octant spectrum, 1/(2N)^3 folded in
     const float* ghat32 = nullptr;
+    const double* gmix64 = nullptr;   // mixed spectrum of the direct i pass, 1/(2N)^2 folded in
+    const float* gmix32 = nullptr;
     const double2* tw64 = nullptr;    // exp(-2 pi i m / 2N); null if not built yet
     const float2* tw32 = nullptr;
 };

@@ -382,7 +382,37 @@ bool periodic_spectrum_applies(int N, double s) {
     return std::pow(2.0 * N, 3) * std::exp(-mu * N) < 1e-14;
 }
 
-void lgf_spectrum(int N, double s, double scale, double* g64, float* g32, cudaStream_t st) {
+// The mixed spectrum of the direct i pass: mix[d][jj][kk], d < N, from the
+// cube transformed along the second and third axes (rows of N + 1 planes)
+__global__ void k_mixed_out(const double* in, long long n, double scale, double* m64, float* m32) {
+    for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < n; x += (long long)gridDim.x * blockDim.x) {
+        const double v = in[x] * scale;
+        m64[x] = v;
+        m32[x] = (float)v;
+    }
+}
+
+// The mixed spectrum of the (2N)-periodic Green's function in closed form:
+// with c = 6 + s - 2 cos(pi jj / N) - 2 cos(pi kk / N) = lam + 1/lam, lam < 1,
+// the inverse transform of 1 / (c - 2 cos(pi p / N)) along p is
+// (lam^d + lam^(2N-d)) / ((1/lam - lam) (1 - lam^2N)). c - 2 is summed from
+// its small terms, so nothing cancels.
+__global__ void k_periodic_mixed(int N, double s, double scale, double* m64, float* m32) {
+    const long long N1 = N + 1, n = N * N1 * N1;
+    for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < n; x += (long long)gridDim.x * blockDim.x) {
+        const int d = (int)(x / (N1 * N1)), j = (int)((x / N1) % N1), k = (int)(x % N1);
+        const double sj = sinpi(0.5 * j / N), sk = sinpi(0.5 * k / N);
+        const double c2 = s + 4.0 * (sj * sj + sk * sk);      // c - 2
+        const double r = sqrt(c2 * (c2 + 4.0));               // 1/lam - lam
+        const double lam = 2.0 / (c2 + 2.0 + r);
+        const double v = scale * (pow(lam, (double)d) + pow(lam, (double)(2 * N - d))) / (r * (1.0 - pow(lam, 2.0 * N)));
+        m64[x] = v;
+        m32[x] = (float)v;
+    }
+}
+
+void lgf_spectrum(int N, double s, double scale, double* g64, float* g32, cudaStream_t st, double mix_scale,
+                  double* mix64, float* mix32) {
     BAE_REQUIRE(is_pow2(N) && N >= 8 && N <= 256, BAE_ERR_INVALID_ARG,
                 "lgf_spectrum: N must be a power of two in [8, 256]");
     BAE_REQUIRE(std::isfinite(s) && s >= 0.0, BAE_ERR_INVALID_ARG, "lgf_spectrum: s must be finite and >= 0");
@@ -394,6 +424,10 @@ void lgf_spectrum(int N, double s, double scale, double* g64, float* g32, cudaSt
         BAE_LAUNCH("k_periodic_spectrum", st,
                    k_periodic_spectrum<<<(int)std::min<long long>((n3 + 255) / 256, 152LL * 16), 256, 0, st>>>(
                        N, s, scale, g64, g32));
+        if (mix64)
+            BAE_LAUNCH("k_periodic_mixed", st,
+                       k_periodic_mixed<<<(int)std::min<long long>((n3 + 255) / 256, 152LL * 16), 256, 0, st>>>(
+                           N, s, mix_scale, mix64, mix32));
         BAE_CUDA(cudaStreamSynchronize(st));
         return;
     }
@@ -410,6 +444,10 @@ void lgf_spectrum(int N, double s, double scale, double* g64, float* g32, cudaSt
     BAE_LAUNCH("k_cos_pass", st, k_cos_pass<<<blocks, 256, smem, st>>>(c0.p, c1.p, Cm.p, N, nlines, 1, N1, nlines, 0));
     // axis 2: line = (i, k), base = i * N1^2 + k, element stride N1
     BAE_LAUNCH("k_cos_pass", st, k_cos_pass<<<blocks, 256, smem, st>>>(c1.p, c0.p, Cm.p, N, nlines, N1, 1, N1, N1 * N1));
+    if (mix64)
+        BAE_LAUNCH("k_mixed_out", st,
+                   k_mixed_out<<<(int)std::min<long long>((n3 + 255) / 256, 152LL * 16), 256, 0, st>>>(
+                       c0.p, N * N1 * N1, mix_scale, mix64, mix32));
     // axis 1: line = (j, k), base = j * N1 + k, element stride N1^2
     BAE_LAUNCH("k_cos_pass", st, k_cos_pass<<<blocks, 256, smem, st>>>(c0.p, c1.p, Cm.p, N, nlines, N1 * N1, 1, nlines, 0));
     BAE_LAUNCH("k_scale_out", st, k_scale_out<<<(int)std::min<long long>((n3 + 255) / 256, 152LL * 16), 256, 0, st>>>(c1.p, n3, scale, g64, g32));

@@ -76,10 +76,12 @@ void apply_into(const ProblemView& pv, const double* q, double* v, unsigned char
     a.B = reinterpret_cast<C*>(scratch + bytes_A);
     if constexpr (sizeof(T) == 8) {
         a.ghat = reinterpret_cast<const T*>(pv.ghat64);
+        a.gmix = reinterpret_cast<const T*>(pv.gmix64);
         a.tw = reinterpret_cast<const C*>(pv.tw64);
         a.v = reinterpret_cast<T*>(v);                          // straight into the caller's output
     } else {
         a.ghat = reinterpret_cast<const T*>(pv.ghat32);
+        a.gmix = reinterpret_cast<const T*>(pv.gmix32);
         a.tw = reinterpret_cast<const C*>(pv.tw32);
         a.v = reinterpret_cast<T*>(scratch + bytes_A + bytes_B);
     }
