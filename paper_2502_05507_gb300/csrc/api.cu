@@ -263,12 +263,13 @@ struct SpectrumCache {
                 box_spectrum(N, s, 1.0 / (L * L * L), sp->g64, sp->g32, st);
                 to_dsf(sp->g64, n3, sp->gds, st);
             } else {
-                const long long nm = (long long)N * (N + 1) * (N + 1);
+                const long long nm = mix_size(N);
                 alloc_check(nm * sizeof(double));
                 BAE_CUDA(cudaMalloc(&sp->m64, nm * sizeof(double)));
                 BAE_CUDA(cudaMalloc(&sp->m32, nm * sizeof(float)));
                 BAE_CUDA(cudaMalloc(&sp->mds, nm * sizeof(dsf)));
                 sp->bytes += nm * (sizeof(double) + sizeof(float) + sizeof(dsf));
+                BAE_CUDA(cudaMemsetAsync(sp->m64, 0, nm * sizeof(double), st));   // the places between the rows
                 lgf_spectrum(N, s, 1.0 / (L * L * L), sp->g64, sp->g32, st, 1.0 / (L * L), sp->m64, sp->m32);
                 to_dsf(sp->m64, nm, sp->mds, st);
                 to_dsf(sp->g64, n3, sp->gds, st);
@@ -339,11 +340,12 @@ struct bae_ctx {
         auto it = tw.find(L);
         if (it != tw.end()) return it->second;
         Twiddles t;
-        t.tw64 = dev_alloc_n<double2>(L, stream);
-        t.tw32 = dev_alloc_n<float2>(L, stream);
-        t.twds = dev_alloc_n<dsc>(L, stream);
+        const int n = 3 * L;   // the tables of length L and L / 2
+        t.tw64 = dev_alloc_n<double2>(n, stream);
+        t.tw32 = dev_alloc_n<float2>(n, stream);
+        t.twds = dev_alloc_n<dsc>(n, stream);
         make_twiddles(L, t.tw64, t.tw32, stream);
-        to_dsf(reinterpret_cast<const double*>(t.tw64), 2LL * L, reinterpret_cast<dsf*>(t.twds), stream);
+        to_dsf(reinterpret_cast<const double*>(t.tw64), 2LL * n, reinterpret_cast<dsf*>(t.twds), stream);
         return tw[L] = t;
     }
 
@@ -772,8 +774,9 @@ void gmres(bae_problem* P, int prec, int nb, const std::vector<int>& which, cons
     // any capture (nothing may allocate or configure inside it)
     // and let the autotuner pick the convolution schedule for this batch size
     // on an uncaptured apply (its result is discarded)
-    const bool tuned = prec == BAE_FP32 ? conv_tuned<float>(P->geo.N, nb)
-                       : prec == BAE_DF64 ? conv_tuned<dsf>(P->geo.N, nb) : conv_tuned<double>(P->geo.N, nb);
+    const bool tuned = prec == BAE_FP32   ? conv_tuned(conv_args<float>(P, nb, true))
+                       : prec == BAE_DF64 ? conv_tuned(conv_args<dsf>(P, nb, true))
+                                          : conv_tuned(conv_args<double>(P, nb, true));
     if (!tuned) apply_rows_prec(P, prec, nb, rhs, n, nullptr, 0, nullptr, ws.tmp.need((long long)nb * n));
     if (prec == BAE_FP32) {
         conv_args<float>(P, nb);

@@ -21,6 +21,14 @@ struct SrcRecipe {
     bool wide = false;
 };
 
+// Place of entry (d, a, b) of the mixed spectrum: rows of N + 1 values, b = 1
+// on a 16-byte boundary (the middle pass of the even-odd schedule copies b =
+// 1..N in 16-byte pieces).
+__host__ __device__ __forceinline__ long long mix_index(int N, int d, int a, int b) {
+    return ((long long)d * (N + 1) + a) * (N + 4) + b + 3;
+}
+inline long long mix_size(int N) { return (long long)N * (N + 1) * (N + 4); }
+
 enum SourceMode { SRC_DENSITY = 0, SRC_VOLUME = 1 };
 
 template <typename T>
@@ -58,10 +66,10 @@ struct ConvArgs {
     cplx_t<T>* B = nullptr;
     const T* ghat = nullptr;      // (N+1)^3 octant, includes 1/(2N)^3
     // the spectrum before its transform along the first axis (direct i pass):
-    // gmix[d][jj][kk], offset d < N, jj, kk <= N, includes 1/(2N)^2 (null:
-    // the i pass is always the FFT)
+    // gmix[d][jj][kk], offset d < N, jj, kk <= N, includes 1/(2N)^2, at
+    // mix_index (null: the i pass is always the FFT)
     const T* gmix = nullptr;
-    const cplx_t<T>* tw = nullptr;  // exp(-2 pi i m / 2N), m < 2N
+    const cplx_t<T>* tw = nullptr;  // twiddle tables of length 2N, then of length N (make_twiddles)
     typename OutOf<T>::type* v = nullptr;   // [nbatch][N^3] output potential
     // x-planes [p0, p1) hold every nonzero source and every output the
     // caller reads (p1 == 0: all N planes). Planes outside are skipped: their
@@ -107,6 +115,16 @@ void run_conv(const ConvArgs<T>& a, cudaStream_t st);
 template <typename T, int L>
 void conv_configure();
 
+// The even-odd schedule (conv_eo.cuh, compiled in conv_eo_*.cu) where its rows
+// fit in shared memory: eo_runs says whether an apply takes it (by the type,
+// L and the plane range alone), eo_apply runs it or returns false.
+template <typename T, int L>
+bool eo_runs(const ConvArgs<T>& a);
+template <typename T, int L>
+bool eo_apply(const ConvArgs<T>& a, cudaStream_t st);
+template <typename T, int L>
+void eo_configure();
+
 // The i pass as a direct sum (conv_direct_*.cu), in place in B.
 template <typename T>
 void launch_direct_i(const ConvArgs<T>& a, cudaStream_t st);
@@ -125,10 +143,11 @@ void cplane_launch(const ConvArgs<T>& a, cudaStream_t st, bool inverse);
 template <typename T>
 void conv_prepare(int N);
 
-// Whether the schedule for (element type, N, batch size) has been chosen
-// already (an apply outside graph capture chooses it by timing both).
+// Whether the schedule of this apply is known: fixed by its plane range or
+// by bae_set_conv_schedule, or chosen already for (element type, N, batch
+// size) (an apply outside graph capture chooses it by timing them).
 template <typename T>
-bool conv_tuned(int N, int nbatch);
+bool conv_tuned(const ConvArgs<T>& a);
 
 // out[b][r] = t[r] v[b][gm[r]] + (1 - t[r]) v[b][partner[r]]  (items with
 // active[b] == 0 skipped when active is not null)

@@ -8,7 +8,7 @@
 #include <string>
 #include <type_traits>
 
-#include "conv.cuh"
+#include "conv_geo.cuh"
 #include "conv_tune.cuh"
 
 namespace bae {
@@ -83,18 +83,6 @@ void tune_store(const std::string& key, int sched) {
 }
 
 namespace {
-
-template <typename T>
-const char* tname() {
-    if constexpr (std::is_same<T, dsf>::value) return "df64";
-    return sizeof(T) == 4 ? "f32" : "f64";
-}
-
-template <typename T>
-const char* kname(const char* f32, const char* f64, const char* ds) {
-    if constexpr (std::is_same<T, dsf>::value) return ds;
-    return sizeof(T) == 4 ? f32 : f64;
-}
 
 
 // ------------------------------------------------------------------ gathers
@@ -187,9 +175,19 @@ void conv_apply(const ConvArgs<T>& a, cudaStream_t st) {
 }
 
 template <typename T>
-bool conv_tuned(int N, int nbatch) {
+bool conv_tuned(const ConvArgs<T>& a) {
     if (forced_sched() >= 0) return true;
-    const std::string key = std::string(tname<T>()) + "/N" + std::to_string(N) + "/nb" + std::to_string(nbatch);
+    bool eo = false;
+    switch (a.N) {
+        case 8: eo = eo_runs<T, 16>(a); break;
+        case 16: eo = eo_runs<T, 32>(a); break;
+        case 32: eo = eo_runs<T, 64>(a); break;
+        case 64: eo = eo_runs<T, 128>(a); break;
+        case 128: eo = eo_runs<T, 256>(a); break;
+        case 256: eo = eo_runs<T, 512>(a); break;
+    }
+    if (eo) return true;
+    const std::string key = std::string(tname<T>()) + "/N" + std::to_string(a.N) + "/nb" + std::to_string(a.nbatch);
     return tune_lookup(key) >= 0;
 }
 
@@ -259,9 +257,9 @@ void to_dsf(const double* in, long long n, dsf* out, cudaStream_t st) {
 template void conv_apply<float>(const ConvArgs<float>&, cudaStream_t);
 template void conv_apply<double>(const ConvArgs<double>&, cudaStream_t);
 template void conv_apply<dsf>(const ConvArgs<dsf>&, cudaStream_t);
-template bool conv_tuned<float>(int, int);
-template bool conv_tuned<double>(int, int);
-template bool conv_tuned<dsf>(int, int);
+template bool conv_tuned<float>(const ConvArgs<float>&);
+template bool conv_tuned<double>(const ConvArgs<double>&);
+template bool conv_tuned<dsf>(const ConvArgs<dsf>&);
 template void conv_prepare<float>(int);
 template void conv_prepare<double>(int);
 template void conv_prepare<dsf>(int);

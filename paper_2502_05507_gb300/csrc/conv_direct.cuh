@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(DirTile<T>::MAXW * 32) k_direct_i(ConvArgs<T> 
     const int b = blockIdx.y;
     T* gs = reinterpret_cast<T*>(smem_raw);                         // [n][32]
     unsigned char* xraw = smem_raw + (size_t)n * 32 * sizeof(T);    // n even: a multiple of 256 bytes
-    const long long dstride = (long long)N1 * N1;                   // entries g(d) and g(d + 1) apart
+    const long long dstride = mix_index(N, 1, 0, 0) - mix_index(N, 0, 0, 0);   // entries g(d) and g(d + 1) apart
     const long long istride = (long long)(2 * N) * N1;              // planes of B apart
     C* Bb = a.B + (long long)b * N * istride + (long long)p0 * istride;
 
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(DirTile<T>::MAXW * 32) k_direct_i(ConvArgs<T> 
         const bool on = pair <= N && kk != 0;
         const bool two = on && pair != 0 && pair != N;   // 2N - jj is another pencil
         // the entries first: they do not depend on the kernel before
-        const T* g = a.gmix + (on ? (long long)pair * N1 + kk : 0);
+        const T* g = a.gmix + (on ? mix_index(N, 0, pair, kk) : 0);
         for (int d = warp; d < n; d += nwarp) gs[d * 32 + lane] = g[min(d, n0 - 1) * dstride];
         wait_prior_grid();
         if (a.active && !a.active[b]) return;   // whole CTA
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(DirTile<T>::MAXW * 32) k_direct_i(ConvArgs<T> 
         const int slot = on ? c >> 1 : 0, comp = c & 1;
         const int jj = slot <= N ? slot : 2 * N - slot;
         const int kn = (slot > N || ((slot == 0 || slot == N) && comp)) ? N : 0;
-        const T* g = a.gmix + (long long)jj * N1 + kn;
+        const T* g = a.gmix + mix_index(N, 0, jj, kn);
         for (int d = warp; d < n; d += nwarp) gs[d * 32 + lane] = g[min(d, n0 - 1) * dstride];
         wait_prior_grid();
         if (a.active && !a.active[b]) return;   // whole CTA

@@ -1,0 +1,10 @@
+// The even-odd schedule for float64, transform length 128.
+#include "conv_eo.cuh"
+
+namespace bae {
+
+template bool eo_runs<double, 128>(const ConvArgs<double>&);
+template bool eo_apply<double, 128>(const ConvArgs<double>&, cudaStream_t);
+template void eo_configure<double, 128>();
+
+}  // namespace bae

@@ -176,6 +176,14 @@ void launch_pdl(K kernel, dim3 grid, int threads, size_t smem, cudaStream_t st, 
     BAE_CUDA(cudaLaunchKernelEx(&cfg, kernel, a...));
 }
 
+// The forms of the even-odd schedule (conv_eo.cuh) per type and length: rows
+// of all 2N frequencies (not for the 16-byte elements at L = 512, whose rows
+// take 8 KB each), and rows split into the even and odd frequencies.
+template <typename T, int L> struct EoUse {
+    static constexpr bool whole = L <= 256 || std::is_same<T, float>::value;
+    static constexpr bool split = L >= 128;
+};
+
 // ------------------------------------------------ packed Nyquist column
 // The k-spectrum of a real line is real at kk = 0 and at kk = N, so both
 // live in column 0 as X0 + i XN and every pass after the k transform runs

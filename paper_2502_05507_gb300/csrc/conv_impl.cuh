@@ -787,6 +787,7 @@ void run_conv(const ConvArgs<T>& a, cudaStream_t st) {
         launch_sched<T, L>(a, st, SCHED_PASSES);
         return;
     }
+    if (forced_sched() < 0 && eo_apply<T, L>(a, st)) return;
     using PG = PlaneGeo<T, L>;
     // the schedules this (element type, L) can run: the five passes, their
     // variant geometry, the plane-fused passes (one CTA, or a cluster)
@@ -844,6 +845,7 @@ void run_conv(const ConvArgs<T>& a, cudaStream_t st) {
 template <typename T, int L>
 void conv_configure() {
     configure_conv<T, L>();
+    eo_configure<T, L>();
 }
 
 }  // namespace bae

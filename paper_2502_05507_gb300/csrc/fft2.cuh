@@ -188,6 +188,14 @@ __device__ __forceinline__ void rdft_zhi(C* v) {
     }
 }
 
+// The barrier around an exchange: the CTA's, or (WARP) the warp's where all
+// threads of a line are in one warp.
+template <bool WARP>
+__device__ __forceinline__ void xch_sync() {
+    if constexpr (WARP) __syncwarp();
+    else __syncthreads();
+}
+
 template <int L> struct Factors;
 template <> struct Factors<16> { static constexpr int R1 = 4, R2 = 4; };
 template <> struct Factors<32> { static constexpr int R1 = 4, R2 = 8; };
@@ -203,32 +211,36 @@ template <> struct Factors<512> { static constexpr int R1 = 16, R2 = 32; };
 
 // n-layout -> k-layout (forward, or inverse when INV: then from the
 // n-layout of X to the k-layout of the inverse transform, same steps with
-// conjugate twiddles). tw: exp(-2 pi i m / L), m < L. ZHI: the input rows
+// conjugate twiddles). tw: exp(-2 pi i m / L), m < L, followed by the table
+// exp(-2 pi i n1 k2 / L) at [k2 R1 + n1], which the threads of a line in one
+// warp (WARP) read at consecutive places and compile-time offsets (the column
+// passes, whose lanes share n1, ran slower with it: 38 against 28 us for the
+// float32 i pass at N = 128). ZHI: the input rows
 // n >= L/2 are zero (v[m] = 0 for m >= R2 / 2).
-template <int L, bool INV, bool ZHI = false, typename C>
+template <int L, bool INV, bool ZHI = false, bool WARP = false, typename C>
 __device__ __forceinline__ void fft_n2k(C* v, C* xch, int base, int sk, int sn, int t, const C* __restrict__ tw) {
     constexpr int R1 = Factors<L>::R1, R2 = Factors<L>::R2, Q = R2 / R1;
     if constexpr (ZHI) rdft_zhi<R2, INV>(v);          // v[k2] = Y[t][k2]
     else rdft<R2, INV>(v);
 #pragma unroll
     for (int k2 = 1; k2 < R2; ++k2) {
-        const C w = ldg_c(tw + t * k2);
+        const C w = ldg_c(WARP ? tw + L + k2 * R1 + t : tw + t * k2);
         v[k2] = INV ? cmulc(v[k2], w) : cmul(v[k2], w);
     }
 #pragma unroll
     for (int k2 = 0; k2 < R2; ++k2) xch[base + k2 * sk + t * sn] = v[k2];
-    __syncthreads();
+    xch_sync<WARP>();
 #pragma unroll
     for (int q = 0; q < Q; ++q)
 #pragma unroll
         for (int n1 = 0; n1 < R1; ++n1) v[q * R1 + n1] = xch[base + (t + q * R1) * sk + n1 * sn];
-    __syncthreads();
+    xch_sync<WARP>();
 #pragma unroll
     for (int q = 0; q < Q; ++q) rdft<R1, INV>(v + q * R1);   // v[q R1 + k1] = X[k2 + R2 k1]
 }
 
 // k-layout -> n-layout (inverse when INV, the mirror of fft_n2k).
-template <int L, bool INV, typename C>
+template <int L, bool INV, bool WARP = false, typename C>
 __device__ __forceinline__ void fft_k2n(C* v, C* xch, int base, int sk, int sn, int t, const C* __restrict__ tw) {
     constexpr int R1 = Factors<L>::R1, R2 = Factors<L>::R2, Q = R2 / R1;
 #pragma unroll
@@ -239,15 +251,16 @@ __device__ __forceinline__ void fft_k2n(C* v, C* xch, int base, int sk, int sn, 
         for (int n1 = 0; n1 < R1; ++n1) {
             const int k2 = t + q * R1;
             if (n1 > 0 && k2 > 0) {
-                const C w = ldg_c(tw + n1 * k2);
+                // (R1 = R2: the table is symmetric, and a warp reads it in order)
+                const C w = ldg_c(WARP ? tw + L + (R1 == R2 ? n1 * R1 + k2 : k2 * R1 + n1) : tw + n1 * k2);
                 v[q * R1 + n1] = INV ? cmulc(v[q * R1 + n1], w) : cmul(v[q * R1 + n1], w);
             }
             xch[base + k2 * sk + n1 * sn] = v[q * R1 + n1];
         }
-    __syncthreads();
+    xch_sync<WARP>();
 #pragma unroll
     for (int k2 = 0; k2 < R2; ++k2) v[k2] = xch[base + k2 * sk + t * sn];
-    __syncthreads();
+    xch_sync<WARP>();
     rdft<R2, INV>(v);                                   // v[n2] = x[t + R1 n2]
 }
 
@@ -272,13 +285,13 @@ struct Plan2 {
     static constexpr int XLEN = L;
     // slot s = q R1 + k1 holds X[t + q R1 + R2 k1]
     __host__ __device__ static constexpr int kidx(int t, int s) { return t + (s / R1) * R1 + R2 * (s % R1); }
-    template <bool ZHI, typename C>
+    template <bool ZHI, bool WARP = false, typename C>
     __device__ __forceinline__ static void fwd(C* v, C* xch, int base, int es, int t, const C* __restrict__ tw) {
-        fft_n2k<L, false, ZHI>(v, xch, base, es == 1 ? R1 + 1 : R1 * es, es, t, tw);
+        fft_n2k<L, false, ZHI, WARP>(v, xch, base, es == 1 ? R1 + 1 : R1 * es, es, t, tw);
     }
-    template <typename C>
+    template <bool WARP = false, typename C>
     __device__ __forceinline__ static void inv(C* v, C* xch, int base, int es, int t, const C* __restrict__ tw) {
-        fft_k2n<L, true>(v, xch, base, es == 1 ? R1 + 1 : R1 * es, es, t, tw);
+        fft_k2n<L, true, WARP>(v, xch, base, es == 1 ? R1 + 1 : R1 * es, es, t, tw);
     }
 };
 
@@ -301,7 +314,8 @@ struct Plan3_512 {
     __host__ __device__ static constexpr int kidx(int t, int s) { return t + 64 * s; }
     __device__ __forceinline__ static int pos(int p) { return p + (p >> 6); }
 
-    template <bool ZHI, typename C>
+    // (the threads of a line are two warps: the barriers are the CTA's)
+    template <bool ZHI, bool = false, typename C>
     __device__ __forceinline__ static void fwd(C* v, C* xch, int base, int es, int t, const C* __restrict__ tw) {
         if constexpr (ZHI) rdft_zhi<8, false>(v);       // v[k3]
         else rdft<8, false>(v);
@@ -327,7 +341,7 @@ struct Plan3_512 {
         rdft<8, false>(v);                               // v[k1] = X[t + 64 k1]
     }
 
-    template <typename C>
+    template <bool = false, typename C>
     __device__ __forceinline__ static void inv(C* v, C* xch, int base, int es, int t, const C* __restrict__ tw) {
         const int c3 = t & 7, c2 = t >> 3;               // this thread's (k3, k2)
         rdft<8, true>(v);                                // v[t1]
@@ -379,7 +393,7 @@ struct Plan3_256 {
         return p ^ (((r & 1) << 2) | (r & 2) | ((r >> 2) & 1));
     }
 
-    template <bool ZHI, typename C>
+    template <bool ZHI, bool WARP = false, typename C>
     __device__ __forceinline__ static void fwd(C* v, C* xch, int base, int es, int t, const C* __restrict__ tw) {
         if constexpr (ZHI) rdft_zhi<8, false>(v);       // v[k3]
         else rdft<8, false>(v);
@@ -387,17 +401,17 @@ struct Plan3_256 {
         for (int k3 = 1; k3 < 8; ++k3) v[k3] = cmul(v[k3], ldg_c(tw + t * k3));
 #pragma unroll
         for (int k3 = 0; k3 < 8; ++k3) xch[base + pos(k3 * 32 + t) * es] = v[k3];
-        __syncthreads();
+        xch_sync<WARP>();
         const int t1 = t & 3, k3 = t >> 2;
 #pragma unroll
         for (int t2 = 0; t2 < 8; ++t2) v[t2] = xch[base + pos(k3 * 32 + t1 + 4 * t2) * es];
-        __syncthreads();
+        xch_sync<WARP>();
         rdft<8, false>(v);                               // v[k2]
 #pragma unroll
         for (int k2 = 1; k2 < 8; ++k2) v[k2] = cmul(v[k2], ldg_c(tw + 8 * t1 * k2));
 #pragma unroll
         for (int k2 = 0; k2 < 8; ++k2) xch[base + pos((k3 * 8 + k2) * 4 + t1) * es] = v[k2];
-        __syncthreads();
+        xch_sync<WARP>();
         const int c3 = t & 7, c2 = t >> 3;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -408,10 +422,10 @@ struct Plan3_256 {
 #pragma unroll
             for (int k1 = 0; k1 < 4; ++k1) v[h + 2 * k1] = w[k1];   // X[t + 32 (h + 2 k1)]
         }
-        __syncthreads();
+        xch_sync<WARP>();
     }
 
-    template <typename C>
+    template <bool WARP = false, typename C>
     __device__ __forceinline__ static void inv(C* v, C* xch, int base, int es, int t, const C* __restrict__ tw) {
         const int c3 = t & 7, c2 = t >> 3;               // this thread's pairs (k3, k2 + 4 h)
 #pragma unroll
@@ -423,20 +437,20 @@ struct Plan3_256 {
 #pragma unroll
             for (int u1 = 0; u1 < 4; ++u1) xch[base + pos((c3 * 8 + c2 + 4 * h) * 4 + u1) * es] = w[u1];
         }
-        __syncthreads();
+        xch_sync<WARP>();
         const int t1 = t & 3, k3 = t >> 2;
 #pragma unroll
         for (int k2 = 0; k2 < 8; ++k2) v[k2] = xch[base + pos((k3 * 8 + k2) * 4 + t1) * es];
-        __syncthreads();
+        xch_sync<WARP>();
 #pragma unroll
         for (int k2 = 1; k2 < 8; ++k2) v[k2] = cmulc(v[k2], ldg_c(tw + 8 * t1 * k2));
         rdft<8, true>(v);                                // v[t2]
 #pragma unroll
         for (int t2 = 0; t2 < 8; ++t2) xch[base + pos(k3 * 32 + t1 + 4 * t2) * es] = v[t2];
-        __syncthreads();
+        xch_sync<WARP>();
 #pragma unroll
         for (int j3 = 0; j3 < 8; ++j3) v[j3] = xch[base + pos(j3 * 32 + t) * es];
-        __syncthreads();
+        xch_sync<WARP>();
 #pragma unroll
         for (int j3 = 1; j3 < 8; ++j3) v[j3] = cmulc(v[j3], ldg_c(tw + t * j3));
         rdft<8, true>(v);                                // v[m] = x[t + 32 m]

@@ -22,6 +22,7 @@
 #include <cmath>
 #include <vector>
 
+#include "conv.cuh"
 #include "lgf.cuh"
 
 namespace bae {
@@ -311,8 +312,22 @@ __global__ void k_twiddles(int L, double2* tw64, float2* tw32) {
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < L; m += gridDim.x * blockDim.x) {
         double sn, cs;
         sincospi(2.0 * (double)m / (double)L, &sn, &cs);
-        if (tw64) tw64[m] = make_double2(cs, -sn);
-        if (tw32) tw32[m] = make_float2((float)cs, (float)-sn);
+        tw64[m] = make_double2(cs, -sn);
+        tw32[m] = make_float2((float)cs, (float)-sn);
+    }
+}
+
+// first thread count of the two-level split of a transform of length L
+// (Factors<L>::R1)
+__host__ __device__ inline int level_one(int L) { return L <= 32 ? 4 : (L <= 128 ? 8 : 16); }
+
+// out[k2 R1 + n1] = exp(-2 pi i n1 k2 / L), n1 < R1, k2 < L / R1
+__global__ void k_twiddle_products(int L, int R1, double2* tw64, float2* tw32) {
+    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < L; x += gridDim.x * blockDim.x) {
+        double sn, cs;
+        sincospi(2.0 * (double)((x % R1) * (x / R1)) / (double)L, &sn, &cs);
+        tw64[x] = make_double2(cs, -sn);
+        tw32[x] = make_float2((float)cs, (float)-sn);
     }
 }
 
@@ -382,13 +397,15 @@ bool periodic_spectrum_applies(int N, double s) {
     return std::pow(2.0 * N, 3) * std::exp(-mu * N) < 1e-14;
 }
 
-// The mixed spectrum of the direct i pass: mix[d][jj][kk], d < N, from the
-// cube transformed along the second and third axes (rows of N + 1 planes)
-__global__ void k_mixed_out(const double* in, long long n, double scale, double* m64, float* m32) {
+// The mixed spectrum of the direct i pass (layout: mix_index) from the cube
+// transformed along the second and third axes
+__global__ void k_mixed_out(const double* in, int N, double scale, double* m64, float* m32) {
+    const long long N1 = N + 1, n = N * N1 * N1;
     for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < n; x += (long long)gridDim.x * blockDim.x) {
+        const long long y = mix_index(N, (int)(x / (N1 * N1)), (int)((x / N1) % N1), (int)(x % N1));
         const double v = in[x] * scale;
-        m64[x] = v;
-        m32[x] = (float)v;
+        m64[y] = v;
+        m32[y] = (float)v;
     }
 }
 
@@ -406,8 +423,9 @@ __global__ void k_periodic_mixed(int N, double s, double scale, double* m64, flo
         const double r = sqrt(c2 * (c2 + 4.0));               // 1/lam - lam
         const double lam = 2.0 / (c2 + 2.0 + r);
         const double v = scale * (pow(lam, (double)d) + pow(lam, (double)(2 * N - d))) / (r * (1.0 - pow(lam, 2.0 * N)));
-        m64[x] = v;
-        m32[x] = (float)v;
+        const long long y = mix_index(N, d, j, k);
+        m64[y] = v;
+        m32[y] = (float)v;
     }
 }
 
@@ -447,7 +465,7 @@ void lgf_spectrum(int N, double s, double scale, double* g64, float* g32, cudaSt
     if (mix64)
         BAE_LAUNCH("k_mixed_out", st,
                    k_mixed_out<<<(int)std::min<long long>((n3 + 255) / 256, 152LL * 16), 256, 0, st>>>(
-                       c0.p, N * N1 * N1, mix_scale, mix64, mix32));
+                       c0.p, N, mix_scale, mix64, mix32));
     // axis 1: line = (j, k), base = j * N1 + k, element stride N1^2
     BAE_LAUNCH("k_cos_pass", st, k_cos_pass<<<blocks, 256, smem, st>>>(c0.p, c1.p, Cm.p, N, nlines, N1 * N1, 1, nlines, 0));
     BAE_LAUNCH("k_scale_out", st, k_scale_out<<<(int)std::min<long long>((n3 + 255) / 256, 152LL * 16), 256, 0, st>>>(c1.p, n3, scale, g64, g32));
@@ -455,7 +473,12 @@ void lgf_spectrum(int N, double s, double scale, double* g64, float* g32, cudaSt
 }
 
 void make_twiddles(int L, double2* tw64, float2* tw32, cudaStream_t st) {
-    BAE_LAUNCH("k_twiddles", st, k_twiddles<<<ceil_div(L, 256), 256, 0, st>>>(L, tw64, tw32));
+    for (int len = L, off = 0; len >= L / 2; off += 2 * len, len /= 2) {
+        BAE_LAUNCH("k_twiddles", st, k_twiddles<<<ceil_div(len, 256), 256, 0, st>>>(len, tw64 + off, tw32 + off));
+        BAE_LAUNCH("k_twiddle_products", st,
+                   k_twiddle_products<<<ceil_div(len, 256), 256, 0, st>>>(len, level_one(len), tw64 + off + len,
+                                                                          tw32 + off + len));
+    }
 }
 
 }  // namespace bae

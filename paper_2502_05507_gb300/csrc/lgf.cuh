@@ -18,8 +18,8 @@ bool periodic_spectrum_applies(int N, double s);
 // ghat[(k1 (N+1) + k2)(N+1) + k3] = sum_n Gemb(n) cos(pi k.n / N), times
 // `scale`. Writes float64 into g64 and, if g32 is not null, float32 into g32.
 // If mix64 is not null, also the mixed spectrum of the direct i pass (float64
-// and float32): mix[(d (N+1) + k2)(N+1) + k3], d < N, the transform along the
-// second and third axes only, times mix_scale.
+// and float32, mix_size values): entry (d, k2, k3), d < N, of the transform
+// along the second and third axes only, times mix_scale, at mix_index.
 void lgf_spectrum(int N, double s, double scale, double* g64, float* g32, cudaStream_t st, double mix_scale = 0.0,
                   double* mix64 = nullptr, float* mix32 = nullptr);
 
@@ -29,7 +29,8 @@ void lgf_spectrum(int N, double s, double scale, double* g64, float* g32, cudaSt
 // the pole (s = 0, k = 0).
 void box_spectrum(int N, double s, double scale, double* g64, float* g32, cudaStream_t st);
 
-// Twiddle tables exp(-2 pi i m / L), m < L, on the device.
+// Twiddle tables on the device, 3 L values: exp(-2 pi i m / L), m < L, and the
+// products table of fft2.cuh for length L (L values), then both for L / 2.
 void make_twiddles(int L, double2* tw64, float2* tw32, cudaStream_t st);
 
 }  // namespace bae

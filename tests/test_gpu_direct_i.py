@@ -41,7 +41,7 @@ SLABS = [(64, 1.2, 0.3), (64, 9.4, 3.0), (64, 18.3, -2.2), (64, 23.9, 0.5), (128
          (128, 29.9, 0.5), (128, 30.4, 1.0), (128, 38.9, 0.0)]
 
 
-@pytest.mark.parametrize("schedule", ["passes"])
+@pytest.mark.parametrize("schedule", ["passes", "auto"])
 @pytest.mark.parametrize("precision", ["fp32", "df64", "fp64"])
 @pytest.mark.parametrize("layer", ["double", "single"])
 @pytest.mark.parametrize("N,half,z0", SLABS)
