@@ -228,7 +228,8 @@ struct SpectrumCache {
     std::mutex mu;
     std::condition_variable cv;
     // key: (N, kind, bit pattern of s); kind 0 = the free-lattice G_s, 1 =
-    // the finite-box Green's function of eq. [aux]
+    // the finite-box Green's function of eq. [aux], 2 = kind 0 for a window of
+    // the grid (no near-field table)
     std::map<std::tuple<int, int, uint64_t>, std::shared_ptr<Spectrum>> map;
     std::set<std::tuple<int, int, uint64_t>> building;
 
@@ -273,9 +274,11 @@ struct SpectrumCache {
                 lgf_spectrum(N, s, 1.0 / (L * L * L), sp->g64, sp->g32, st, 1.0 / (L * L), sp->m64, sp->m32);
                 to_dsf(sp->m64, nm, sp->mds, st);
                 to_dsf(sp->g64, n3, sp->gds, st);
-                alloc_check(NEAR_TAB * sizeof(double));
-                BAE_CUDA(cudaMalloc(&sp->near, NEAR_TAB * sizeof(double)));
-                lgf_table(NEAR_TN, s, sp->near, st);
+                if (kind == 0) {
+                    alloc_check(NEAR_TAB * sizeof(double));
+                    BAE_CUDA(cudaMalloc(&sp->near, NEAR_TAB * sizeof(double)));
+                    lgf_table(NEAR_TN, s, sp->near, st);
+                }
             }
             BAE_CUDA(cudaStreamSynchronize(st));
         } catch (...) {
@@ -352,11 +355,47 @@ struct bae_ctx {
     std::shared_ptr<Spectrum> spectrum(int N, double s, int kind = 0) { return cache->get(N, s, stream, kind); }
 };
 
+// The box of the pruned applies on the grid they run on (the swapped view when
+// there is one): planes [p0, p1), lines [q0, q1) (even bounds), and the
+// window of nt nodes per axis from (w0, w1, w2) that the transforms cover: 3/4
+// of the grid where the box fits it (N >= 64), since a transform of length
+// 3N/2 does all that one of length 2N does for a box of 3N/4 nodes, with 3/4 of
+// the work along each of the three axes. Measured whole grid / window: star at N =
+// 256, 172 planes, float32 apply 461 / 255 us, double-float 1.67 / 1.04 ms; torus
+// at N = 128, 64 right-hand sides, float32 468 / 405 us, double-float 2.77 / 1.88
+// ms. At N = 32 the window's three short stages cost more than they save (float64
+// operator 57 / 74 us).
+struct ConvBox {
+    int p0 = 0, p1 = 0, q0 = 0, q1 = 0;
+    int nt = 0, w0 = 0, w1 = 0, w2 = 0;
+};
+
+static ConvBox conv_box(const Geometry& g) {
+    const int N = g.N, sw = g.cv_swap;
+    const int ax1 = sw == 1 ? 0 : 1, ax2 = sw == 2 ? 0 : 2;
+    ConvBox c;
+    c.p0 = g.src_lo[sw];
+    c.p1 = g.src_hi[sw];
+    c.q0 = g.src_lo[ax1] & ~1;   // whole pairs of lines 2 p, 2 p + 1, in every schedule
+    c.q1 = (g.src_hi[ax1] + 1) & ~1;
+    c.nt = N;
+    const int nw = 3 * N / 4;
+    if (N >= 64 && c.p1 - c.p0 <= nw && c.q1 - c.q0 <= nw && g.src_hi[ax2] - g.src_lo[ax2] <= nw) {
+        c.nt = nw;
+        c.w0 = std::min(c.p0, N - nw);
+        c.w1 = std::min(c.q0, N - nw);
+        c.w2 = std::min(g.src_lo[ax2], N - nw);
+    }
+    return c;
+}
+
 struct bae_problem {
     bae_ctx* ctx = nullptr;
     Geometry geo;
     Precond pre;   // right preconditioner, built on the first mixed solve that asks for it
     std::shared_ptr<Spectrum> spec;
+    ConvBox box;                          // planes and window of the pruned applies
+    std::shared_ptr<Spectrum> spec_win;   // spectrum of the window's size, when it is smaller than the grid
     std::shared_ptr<Spectrum> spec_box;   // finite-box spectrum, fetched by the first box apply
     double kappa2 = 0.0, s = 0.0;
     // direct formulation: the Arnoldi gather reads the operator rows as they
@@ -414,39 +453,50 @@ const int* partner_of(const bae_problem* P, bool pruned) {
 int swap_of(const bae_problem* P, bool pruned) { return use_view(P, pruned) ? P->geo.cv_swap : 0; }
 
 template <typename T>
-ConvArgs<T> conv_args(bae_problem* P, int nb, bool pruned = false) {
+ConvArgs<T> conv_args(bae_problem* P, int nb, bool pruned = false, bool windowed = true) {
     const int N = P->geo.N;
     const long long N1 = N + 1;
     ConvArgs<T> a;
-    a.N = N;
+    a.N = a.nt = N;
     a.nbatch = nb;
     const bool view = use_view(P, pruned);
+    const Spectrum* spec = P->spec.get();
     if (pruned) {
-        a.p0 = view ? P->geo.cv_lo : P->geo.plane_lo;
-        a.p1 = view ? P->geo.cv_hi : P->geo.plane_hi;
-        // the line range along the grid's second axis (y, or x when x and
-        // y are swapped), rounded out to whole line pairs
-        const int ax2 = (view && P->geo.cv_swap == 1) ? 0 : 1;
-        a.q0 = P->geo.ext_lo[ax2] & ~1;
-        a.q1 = std::min(N, (P->geo.ext_hi[ax2] + 1) & ~1);
+        const ConvBox& c = P->box;
+        a.p0 = c.p0;
+        a.p1 = c.p1;
+        a.q0 = c.q0;
+        a.q1 = c.q1;
+        // (a schedule set by bae_set_conv_schedule runs on the whole grid)
+        if (windowed && P->spec_win && forced_sched() < 0) {
+            spec = P->spec_win.get();
+            a.nt = c.nt;
+            a.w0 = c.w0;
+            a.w1 = c.w1;
+            a.w2 = c.w2;
+            a.p0 -= c.w0;
+            a.p1 -= c.w0;
+            a.q0 -= c.w1;
+            a.q1 -= c.w1;
+        }
     }
     a.rec = view ? P->geo.cv_recipe() : P->geo.recipe();
     a.flags = view ? P->geo.cv_flags : P->geo.flags;
     a.f_swap = swap_of(P, pruned);
     a.A = reinterpret_cast<cplx_t<T>*>(P->ws().A.need((long long)nb * N * N * N1));
     a.B = reinterpret_cast<cplx_t<T>*>(P->ws().B.need((long long)nb * N * 2 * N * N1));
-    const Twiddles& tw = P->ctx->twiddles(2 * N);
+    const Twiddles& tw = P->ctx->twiddles(2 * a.nt);
     if constexpr (std::is_same<T, dsf>::value) {
-        a.ghat = P->spec->gds;
-        a.gmix = P->spec->mds;
+        a.ghat = spec->gds;
+        a.gmix = spec->mds;
         a.tw = tw.twds;
     } else if constexpr (sizeof(T) == 8) {
-        a.ghat = reinterpret_cast<const T*>(P->spec->g64);
-        a.gmix = reinterpret_cast<const T*>(P->spec->m64);
+        a.ghat = reinterpret_cast<const T*>(spec->g64);
+        a.gmix = reinterpret_cast<const T*>(spec->m64);
         a.tw = reinterpret_cast<const cplx_t<T>*>(tw.tw64);
     } else {
-        a.ghat = reinterpret_cast<const T*>(P->spec->g32);
-        a.gmix = reinterpret_cast<const T*>(P->spec->m32);
+        a.ghat = reinterpret_cast<const T*>(spec->g32);
+        a.gmix = reinterpret_cast<const T*>(spec->m32);
         a.tw = reinterpret_cast<const cplx_t<T>*>(tw.tw32);
     }
     return a;
@@ -492,7 +542,7 @@ template <typename T>
 out_t<T>* apply_box(bae_problem* P, int nb, const double* f, double scale, bool pruned) {
     static_assert(sizeof(T) == 8, "the finite-box apply is float64-accurate");
     if (!P->spec_box) P->spec_box = P->ctx->spectrum(P->geo.N, P->s, 1);
-    ConvArgs<T> a = conv_args<T>(P, nb, pruned);
+    ConvArgs<T> a = conv_args<T>(P, nb, pruned, false);
     if constexpr (std::is_same<T, dsf>::value) a.ghat = P->spec_box->gds;
     else a.ghat = reinterpret_cast<const T*>(P->spec_box->g64);
     a.mode = SRC_VOLUME;
@@ -781,15 +831,15 @@ void gmres(bae_problem* P, int prec, int nb, const std::vector<int>& which, cons
     if (prec == BAE_FP32) {
         conv_args<float>(P, nb);
         vbuf<float>(P, nb);
-        conv_prepare<float>(P->geo.N);
+        conv_prepare<float>(conv_args<float>(P, nb, true).nt);
     } else if (prec == BAE_DF64) {
         conv_args<dsf>(P, nb);
         vbuf<dsf>(P, nb);
-        conv_prepare<dsf>(P->geo.N);
+        conv_prepare<dsf>(conv_args<dsf>(P, nb, true).nt);
     } else {
         conv_args<double>(P, nb);
         vbuf<double>(P, nb);
-        conv_prepare<double>(P->geo.N);
+        conv_prepare<double>(conv_args<double>(P, nb, true).nt);
     }
 
     // a graph captured by an earlier call with the same values is replayed
@@ -1560,6 +1610,11 @@ int bae_problem_create(bae_ctx* ctx, int N, double h, const double origin[3], co
         try {
             P->spec = ctx->spectrum(N, P->s);
             ctx->twiddles(2 * N);   // built here so that later applies allocate nothing
+            P->box = conv_box(P->geo);
+            if (P->box.nt != N) {
+                P->spec_win = ctx->spectrum(P->box.nt, P->s, 2);
+                ctx->twiddles(2 * P->box.nt);
+            }
         // the Schwarz rows of the default (mixed, preconditioned) solve, built
         // on the side stream from here on; a solve waits for them only when it
         // uses them

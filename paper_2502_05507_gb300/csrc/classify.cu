@@ -16,7 +16,7 @@ namespace bae {
 
 namespace {
 
-constexpr int SCAN_E = 8;   // entries per thread of the line-count scans
+constexpr int SCAN_E = 16;   // entries per thread of the line-count scans
 
 __constant__ int c_dir[6][3] = {{1, 0, 0}, {-1, 0, 0}, {0, 1, 0}, {0, -1, 0}, {0, 0, 1}, {0, 0, -1}};
 
@@ -55,29 +55,46 @@ __device__ int block_exclusive_scan(int v, int* s_warp) {
 constexpr int LINE_T = 128;
 
 // slots of the small device record the host reads once
-enum { I_ERR = 0, I_GP, I_MP, I_FIRST, I_LAST, I_NGM, I_NSRC, I_NTERM, I_NGPL, I_FIRSTY, I_LASTY, I_FIRSTZ, I_LASTZ,
+// (I_NGM .. I_MP: the totals of the scans, in the order of their arrays)
+enum { I_ERR = 0, I_FIRST, I_LAST, I_NGM, I_NSRC, I_NTERM, I_GP, I_MP, I_FIRSTY, I_LASTY, I_FIRSTZ, I_LASTZ,
        I_COUNT };
 
 __device__ __forceinline__ bool in_grid(int i, int j, int k, int N) {
     return (unsigned)i < (unsigned)N && (unsigned)j < (unsigned)N && (unsigned)k < (unsigned)N;
 }
 
+// phi < 0 and phi not finite, by integer operations: a float64 comparison
+// holds GB300's FP64 pipe for 64 cycles per warp, and seven of them per node
+// were what k_nbits took (N = 128: 42 us)
+__device__ __forceinline__ bool negative(double p) {
+    const int hi = __double2hiint(p);
+    return hi < 0 && (((hi & 0x7fffffff) | __double2loint(p)) != 0);
+}
+__device__ __forceinline__ bool not_finite(double p) { return (__double2hiint(p) & 0x7ff00000) == 0x7ff00000; }
+
+// atomicMax, left out where the value is there already (a stale read only
+// costs the atomic): thousands of lines raise the same few maxima
+__device__ __forceinline__ void raise(int* m, int v) {
+    if (*reinterpret_cast<volatile int*>(m) < v) atomicMax(m, v);
+}
+
 // bits per node from phi: bit0 in M+ (phi < 0), bit1 an M+ neighbour, bit2
-// a neighbour outside M+ (nodes outside the box count as exterior)
+// a neighbour outside M+ (nodes outside the box count as exterior); a phi that
+// is not finite ends the problem, whatever its bits
 __global__ void __launch_bounds__(LINE_T) k_nbits(const double* __restrict__ phi, int N, uint8_t* __restrict__ nb,
                                                  int* __restrict__ info) {
     const int line = blockIdx.x, i = line / N, j = line - i * N;
     const long long base = (long long)line * N;
     for (int k = threadIdx.x; k < N; k += blockDim.x) {
         const double p = phi[base + k];
-        if (!isfinite(p)) atomicOr(info + I_ERR, 1);
+        if (not_finite(p)) atomicOr(info + I_ERR, 1);
         bool h = false, e = false;
         for (int d = 0; d < 6; ++d) {
             const int ii = i + c_dir[d][0], jj = j + c_dir[d][1], kk = k + c_dir[d][2];
-            if (in_grid(ii, jj, kk, N) && phi[((long long)ii * N + jj) * N + kk] < 0.0) h = true;
+            if (in_grid(ii, jj, kk, N) && negative(phi[((long long)ii * N + jj) * N + kk])) h = true;
             else e = true;
         }
-        nb[base + k] = (uint8_t)((p < 0.0 ? 1 : 0) | (h ? 2 : 0) | (e ? 4 : 0));
+        nb[base + k] = (uint8_t)((negative(p) ? 1 : 0) | (h ? 2 : 0) | (e ? 4 : 0));
     }
 }
 
@@ -88,13 +105,12 @@ __global__ void __launch_bounds__(LINE_T) k_nbits(const double* __restrict__ phi
 // N+ (bits 4-6). Per line: the gamma- nodes, the sources (flags & src_mask)
 // and their stencil terms (a D-node: one per gamma- neighbour; a gamma- node:
 // 1, or with `direct` 1 + its neighbours in gamma = gamma- u gamma+), the
-// gamma+ nodes; M+ and gamma+ totals and the range of source planes go to
-// info.
+// gamma+ nodes, the M+ nodes; the range of source planes goes to info.
 __global__ void __launch_bounds__(LINE_T) k_flags_lines(const uint8_t* __restrict__ nb, int N, int src_mask,
                                                        bool direct, uint8_t* __restrict__ flags,
                                                        int* __restrict__ cnt_gm, int* __restrict__ cnt_src,
                                                        int* __restrict__ cnt_term, int* __restrict__ cnt_gp,
-                                                       int* __restrict__ info) {
+                                                       int* __restrict__ cnt_mp, int* __restrict__ info) {
     __shared__ int s_red[5][LINE_T / 32];
     const int line = blockIdx.x, i = line / N, j = line - i * N;
     const long long base = (long long)line * N;
@@ -139,8 +155,8 @@ __global__ void __launch_bounds__(LINE_T) k_flags_lines(const uint8_t* __restric
     klo = __reduce_min_sync(0xffffffffu, klo);
     khi = __reduce_max_sync(0xffffffffu, khi);
     if (lane == 0 && khi >= 0) {
-        atomicMax(info + I_FIRSTZ, N - klo);
-        atomicMax(info + I_LASTZ, khi + 1);
+        raise(info + I_FIRSTZ, N - klo);
+        raise(info + I_LASTZ, khi + 1);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -151,45 +167,54 @@ __global__ void __launch_bounds__(LINE_T) k_flags_lines(const uint8_t* __restric
         cnt_src[line] = t[1];
         cnt_term[line] = t[2];
         cnt_gp[line] = t[3];
-        if (t[3]) atomicAdd(info + I_GP, t[3]);
-        if (t[4]) atomicAdd(info + I_MP, t[4]);
+        cnt_mp[line] = t[4];
         if (t[1]) {
-            atomicMax(info + I_FIRST, N - i);
-            atomicMax(info + I_LAST, i + 1);
-            atomicMax(info + I_FIRSTY, N - j);
-            atomicMax(info + I_LASTY, j + 1);
+            raise(info + I_FIRST, N - i);
+            raise(info + I_LAST, i + 1);
+            raise(info + I_FIRSTY, N - j);
+            raise(info + I_LASTY, j + 1);
         }
     }
 }
 
-// In-place exclusive scans of the four per-line counts (nl + 1 entries,
-// the last one becomes the total), one CTA each; totals to info.
-__global__ void __launch_bounds__(1024) k_scan_lines(int* c0, int* c1, int* c2, int* c3, int nl, int* info) {
+// In-place exclusive scans of the per-line counts (nl + 1 entries, the last
+// one becomes the total; nl a multiple of SCAN_E), one CTA each; totals to
+// info.
+__global__ void __launch_bounds__(1024) k_scan_lines(int* c0, int* c1, int* c2, int* c3, int* c4, int nl, int* info) {
     __shared__ int s_warp[33];
     __shared__ int s_carry;
-    int* arr = blockIdx.x == 0 ? c0 : (blockIdx.x == 1 ? c1 : (blockIdx.x == 2 ? c2 : c3));
+    int* arr = blockIdx.x == 0 ? c0 : (blockIdx.x == 1 ? c1 : (blockIdx.x == 2 ? c2 : (blockIdx.x == 3 ? c3 : c4)));
     if (threadIdx.x == 0) s_carry = 0;
     __syncthreads();
-    for (int base = 0; base <= nl; base += blockDim.x * SCAN_E) {
+    for (int base = 0; base < nl; base += blockDim.x * SCAN_E) {
         int v[SCAN_E], tot = 0;
         const int b0 = base + threadIdx.x * SCAN_E;
+        const bool in = b0 < nl;   // all of the thread's entries or none
 #pragma unroll
-        for (int e = 0; e < SCAN_E; ++e) {
-            v[e] = (b0 + e < nl) ? arr[b0 + e] : 0;
-            tot += v[e];
+        for (int e = 0; e < SCAN_E; e += 4) {
+            const int4 q = in ? *reinterpret_cast<const int4*>(arr + b0 + e) : make_int4(0, 0, 0, 0);
+            v[e] = q.x;
+            v[e + 1] = q.y;
+            v[e + 2] = q.z;
+            v[e + 3] = q.w;
+            tot += q.x + q.y + q.z + q.w;
         }
         const int ex = block_exclusive_scan(tot, s_warp);
         int run = ex + s_carry;
 #pragma unroll
-        for (int e = 0; e < SCAN_E; ++e) {
-            if (b0 + e <= nl) arr[b0 + e] = run;
-            run += v[e];
+        for (int e = 0; e < SCAN_E; e += 4) {
+            const int4 q = make_int4(run, run + v[e], run + v[e] + v[e + 1], run + v[e] + v[e + 1] + v[e + 2]);
+            if (in) *reinterpret_cast<int4*>(arr + b0 + e) = q;
+            run = q.w + v[e + 3];
         }
         __syncthreads();
         if (threadIdx.x == 0) s_carry += s_warp[32];
         __syncthreads();
     }
-    if (threadIdx.x == 0) info[I_NGM + blockIdx.x] = s_carry;
+    if (threadIdx.x == 0) {
+        arr[nl] = s_carry;
+        info[I_NGM + blockIdx.x] = s_carry;
+    }
 }
 
 // The lists in lexicographic order: per line, the CTA scans its nodes
@@ -514,8 +539,8 @@ void build_view(Geometry& g, int sw, int src_mask, Scratch& sc, cudaStream_t st)
     BAE_LAUNCH("k_view_count", st,
                k_view_count<<<(unsigned)nl, LINE_T, 0, st>>>(g.cv_flags, N, sw, src_mask, smap, g.term_off, off_src,
                                                              off_term));
-    // blocks 0 and 1 scan the two counts (the other two arrays are not read)
-    BAE_LAUNCH("k_scan_lines", st, k_scan_lines<<<2, 1024, 0, st>>>(off_src, off_term, off_src, off_term, (int)nl, info));
+    // blocks 0 and 1 scan the two counts (the other arrays are not read)
+    BAE_LAUNCH("k_scan_lines", st, k_scan_lines<<<2, 1024, 0, st>>>(off_src, off_term, off_src, off_term, off_src, (int)nl, info));
     g.cv_src_lin = dev_alloc_n<int>(g.n_src, st);
     g.cv_term_off = dev_alloc_n<int>(g.n_src + 1, st);
     int* vorig = sc.get<int>(std::max(1LL, g.n_src));
@@ -576,10 +601,11 @@ void build_geometry(const double* phi, int N, double h, const double origin[3], 
     int* off_gm = sc.get<int>(nl + 1);
     int* off_term = sc.get<int>(nl + 1);
     int* off_gp = sc.get<int>(nl + 1);
+    int* off_mp = sc.get<int>(nl + 1);
     BAE_LAUNCH("k_flags_lines", st,
                k_flags_lines<<<(unsigned)nl, LINE_T, 0, st>>>(nbits, N, src_mask, direct, g.flags, off_gm, g.line_off,
-                                                              off_term, off_gp, info));
-    BAE_LAUNCH("k_scan_lines", st, k_scan_lines<<<4, 1024, 0, st>>>(off_gm, g.line_off, off_term, off_gp, (int)nl, info));
+                                                              off_term, off_gp, off_mp, info));
+    BAE_LAUNCH("k_scan_lines", st, k_scan_lines<<<5, 1024, 0, st>>>(off_gm, g.line_off, off_term, off_gp, off_mp, (int)nl, info));
     int rec[I_COUNT];
     BAE_CUDA(cudaMemcpyAsync(rec, info, sizeof(rec), cudaMemcpyDeviceToHost, st));
     BAE_CUDA(cudaStreamSynchronize(st));
@@ -626,6 +652,8 @@ void build_geometry(const double* phi, int N, double h, const double origin[3], 
     const int slot[3][2] = {{I_FIRST, I_LAST}, {I_FIRSTY, I_LASTY}, {I_FIRSTZ, I_LASTZ}};
     for (int ax = 0; ax < 3; ++ax) {
         const long long first = N - rec[slot[ax][0]], last = rec[slot[ax][1]] - 1;
+        g.src_lo[ax] = (int)first;
+        g.src_hi[ax] = (int)last + 1;
         g.ext_lo[ax] = (int)std::max(0LL, first - 1);
         g.ext_hi[ax] = (int)std::min((long long)N, last + 2);
     }

@@ -34,6 +34,9 @@ struct Geometry {
     int plane_lo = 0, plane_hi = 0;
     // the same range along each axis (0: x, 1: y, 2: z)
     int ext_lo[3] = {0, 0, 0}, ext_hi[3] = {0, 0, 0};
+    // without the plane of margin: the planes that hold sources (gamma- is
+    // among them, and M+ and the partners lie between gamma- nodes)
+    int src_lo[3] = {0, 0, 0}, src_hi[3] = {0, 0, 0};
 
     // Swapped view of the pruned applies: the convolution skips the zero
     // planes of its first axis only, so it runs on the grid with axis 0

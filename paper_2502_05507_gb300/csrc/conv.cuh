@@ -34,6 +34,11 @@ enum SourceMode { SRC_DENSITY = 0, SRC_VOLUME = 1 };
 template <typename T>
 struct ConvArgs {
     int N = 0;
+    // the transforms run on the window of nt^3 nodes that starts at node (w0,
+    // w1, w2) of the grid (in its swapped layout): planes, lines and the
+    // buffers A and B count from the window, recipe, flags, f and v are the
+    // grid's (nt == N: the whole grid)
+    int nt = 0, w0 = 0, w1 = 0, w2 = 0;
     int nbatch = 1;
     SourceMode mode = SRC_DENSITY;
     // SRC_DENSITY: q [nbatch][q_stride] float64 density on gamma-; when q_row
@@ -61,7 +66,8 @@ struct ConvArgs {
     // rec, flags and the output v are in the swapped layout, f in the
     // caller's, so f is read at swap_axes(x) (0: no swap)
     int f_swap = 0;
-    // work buffers (per batch item): A = N*N*(N+1), B = N*2N*(N+1) complex
+    // work buffers (per batch item): A = N*N*(N+1), B = N*2N*(N+1) complex, N
+    // = nt here and in the spectra and twiddles
     cplx_t<T>* A = nullptr;
     cplx_t<T>* B = nullptr;
     const T* ghat = nullptr;      // (N+1)^3 octant, includes 1/(2N)^3
@@ -85,7 +91,7 @@ struct ConvArgs {
     // apply of the same (element type, N, batch size), else the default
     bool no_tune = false;
     __host__ __device__ int plane_lo() const { return p1 > 0 ? p0 : 0; }
-    __host__ __device__ int plane_hi() const { return p1 > 0 ? p1 : N; }
+    __host__ __device__ int plane_hi() const { return p1 > 0 ? p1 : nt; }
     // lines [q0, q1) along the second axis (even bounds) hold every source
     // and every node read back (q1 == 0: all N). The k passes transform
     // only the line pairs of the planes [p0, p1) inside it; the forward j
@@ -93,14 +99,19 @@ struct ConvArgs {
     // them. The plane-fused kernels transform every line.
     int q0 = 0, q1 = 0;
     __host__ __device__ int line_lo() const { return q1 > 0 ? q0 : 0; }
-    __host__ __device__ int line_hi() const { return q1 > 0 ? q1 : N; }
+    __host__ __device__ int line_hi() const { return q1 > 0 ? q1 : nt; }
     __host__ __device__ int pairs_per_plane() const { return (line_hi() - line_lo()) / 2; }
     // line pairs of the k passes, and the first line of pair gp (pairs
     // numbered plane by plane)
     __host__ __device__ long long npairs() const { return (long long)(plane_hi() - plane_lo()) * pairs_per_plane(); }
     __host__ __device__ long long pair_line(long long gp) const {
-        const int npq = pairs_per_plane();
-        return (long long)(plane_lo() + gp / npq) * N + line_lo() + 2 * (gp % npq);
+        const int npq = pairs_per_plane(), g = (int)gp;   // below N^2
+        return (long long)(plane_lo() + g / npq) * nt + line_lo() + 2 * (g % npq);
+    }
+    // the grid's line of line l of the window
+    __host__ __device__ int grid_line(long long l) const {
+        const int i = (int)l / nt;
+        return (i + w0) * N + (int)l - i * nt + w1;
     }
 };
 
@@ -114,6 +125,10 @@ template <typename T, int L>
 void run_conv(const ConvArgs<T>& a, cudaStream_t st);
 template <typename T, int L>
 void conv_configure();
+// the same for an apply on a window of L / 2 = 48, 96 or 192 nodes
+// (conv_window_*.cu)
+template <typename T, int L>
+void run_window(const ConvArgs<T>& a, cudaStream_t st);
 
 // The even-odd schedule (conv_eo.cuh, compiled in conv_eo_*.cu) where its rows
 // fit in shared memory: eo_runs says whether an apply takes it (by the type,
@@ -138,10 +153,11 @@ bool cplane_ready();
 template <typename T, int L>
 void cplane_launch(const ConvArgs<T>& a, cudaStream_t st, bool inverse);
 
-// Sets the kernel attributes conv_apply needs for grid size N (done on the
-// first apply anyway; call it before capturing applies in a CUDA graph).
+// Sets the kernel attributes conv_apply needs for transforms of length 2 nt
+// (done on the first apply anyway; call it before capturing applies in a CUDA
+// graph).
 template <typename T>
-void conv_prepare(int N);
+void conv_prepare(int nt);
 
 // Whether the schedule of this apply is known: fixed by its plane range or
 // by bae_set_conv_schedule, or chosen already for (element type, N, batch

@@ -163,7 +163,10 @@ __global__ void k_widen(const T* v, long long n, double* out) {
 
 template <typename T>
 void conv_apply(const ConvArgs<T>& a, cudaStream_t st) {
-    switch (a.N) {
+    switch (a.nt) {
+        case 48: run_window<T, 96>(a, st); break;
+        case 96: run_window<T, 192>(a, st); break;
+        case 192: run_window<T, 384>(a, st); break;
         case 8: run_conv<T, 16>(a, st); break;
         case 16: run_conv<T, 32>(a, st); break;
         case 32: run_conv<T, 64>(a, st); break;
@@ -177,6 +180,7 @@ void conv_apply(const ConvArgs<T>& a, cudaStream_t st) {
 template <typename T>
 bool conv_tuned(const ConvArgs<T>& a) {
     if (forced_sched() >= 0) return true;
+    if (a.nt != a.N) return true;   // a window: no choice to make
     bool eo = false;
     switch (a.N) {
         case 8: eo = eo_runs<T, 16>(a); break;
@@ -192,8 +196,11 @@ bool conv_tuned(const ConvArgs<T>& a) {
 }
 
 template <typename T>
-void conv_prepare(int N) {
-    switch (N) {
+void conv_prepare(int nt) {
+    switch (nt) {
+        case 48: conv_configure<T, 96>(); break;
+        case 96: conv_configure<T, 192>(); break;
+        case 192: conv_configure<T, 384>(); break;
         case 8: conv_configure<T, 16>(); break;
         case 16: conv_configure<T, 32>(); break;
         case 32: conv_configure<T, 64>(); break;

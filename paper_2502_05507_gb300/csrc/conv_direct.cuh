@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(DirTile<T>::MAXW * 32) k_direct_i(ConvArgs<T> 
     using C = cplx_t<T>;
     constexpr int TI = DirTile<T>::TI;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = a.N, N1 = N + 1;
+    const int N = a.nt, N1 = N + 1;
     const int p0 = a.plane_lo(), n0 = a.plane_hi() - p0;
     const int n = n0 + (n0 & 1), m = n / 2, mb = (m + TI - 1) / TI, mp = mb * TI;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(DirTile<T>::MAXW * 32) k_direct_i(ConvArgs<T> 
 template <typename T>
 void launch_direct_i(const ConvArgs<T>& a, cudaStream_t st) {
     constexpr int TI = DirTile<T>::TI, MAXW = DirTile<T>::MAXW;
-    const int N = a.N, n0 = a.plane_hi() - a.plane_lo();
+    const int N = a.nt, n0 = a.plane_hi() - a.plane_lo();
     const int n = n0 + (n0 & 1), mb = (n / 2 + TI - 1) / TI;
     const int nreg = ceil_div((long long)N * (N + 1), 32), ncol = ceil_div(4 * N, 32);
     const size_t smem = (size_t)n * 32 * sizeof(T) + (size_t)mb * TI * 2 * 4 * 32 * sizeof(T);

@@ -37,6 +37,9 @@ namespace bae {
 template <typename T, int L> struct EoPlan { using type = Plan2<L>; };
 template <> struct EoPlan<double, 256> { using type = Plan3_256; };
 template <> struct EoPlan<dsf, 256> { using type = Plan3_256; };
+template <typename T> struct EoPlan<T, 96> : PlanWin<T, 96> {};
+template <typename T> struct EoPlan<T, 192> : PlanWin<T, 192> {};
+template <typename T> struct EoPlan<T, 384> : PlanWin<T, 384> {};
 template <> struct EoPlan<double, 512> { using type = Plan3_512; };
 template <> struct EoPlan<dsf, 512> { using type = Plan3_512; };
 
@@ -138,7 +141,8 @@ __global__ void __launch_bounds__(EoGeo<T, L>::KT) k_eo_fwd(ConvArgs<T> a, int n
     const bool two = pj < a.plane_hi();                   // the mirrored plane exists
     const int t = threadIdx.x % TH, p = threadIdx.x / TH;
     const bool on = p < cnt;
-    const long long la = (long long)pi * N + q0 + j0, lb = (long long)pj * N + q0 + j0;   // first lines
+    const int NG = a.N;   // the grid's pitch; first lines of the grid:
+    const long long la = (long long)(pi + a.w0) * NG + q0 + j0 + a.w1, lb = (long long)(pj + a.w0) * NG + q0 + j0 + a.w1;
     const T zero = dir_zero(T());
 
     C v[S];
@@ -147,7 +151,7 @@ __global__ void __launch_bounds__(EoGeo<T, L>::KT) k_eo_fwd(ConvArgs<T> a, int n
         for (int k = t; k < 2 * N; k += TH) {
             const bool first = k < N;
             ro[k] = (on && (first || two))
-                        ? volume_or_zero(a, b, ((first ? la : lb) + p) * N + (first ? k : k - N)) : zero;
+                        ? volume_or_zero(a, b, ((first ? la : lb) + p) * NG + a.w2 + (first ? k : k - N)) : zero;
         }
         __syncthreads();
         const double* q = a.q + (long long)b * a.q_stride + (a.q_row ? (long long)a.q_row[b] * a.q_row_stride : 0);
@@ -157,8 +161,8 @@ __global__ void __launch_bounds__(EoGeo<T, L>::KT) k_eo_fwd(ConvArgs<T> a, int n
         for (int e = threadIdx.x; e < na + nb; e += blockDim.x) {
             const bool first = e < na;
             const int s = first ? a0 + e : b0 + e - na;
-            const int x = a.rec.src_lin[s] - (int)((first ? la : lb) * N);   // (line, k) within the CTA's lines
-            rho[(x / N) * G::RS + (first ? 0 : N) + x % N] = source_value<T>(a.rec, s, q, q32);
+            const int x = a.rec.src_lin[s] - (int)((first ? la : lb) * NG);   // (line, k) within the CTA's lines
+            rho[(x / NG) * G::RS + (first ? 0 : N) + x % NG - a.w2] = source_value<T>(a.rec, s, q, q32);
         }
         __syncthreads();
 #pragma unroll
@@ -167,14 +171,14 @@ __global__ void __launch_bounds__(EoGeo<T, L>::KT) k_eo_fwd(ConvArgs<T> a, int n
             v[s] = s < S / 2 ? cmake<C>(ro[x] + ro[N + x], ro[x] - ro[N + x]) : cmake<C>(zero, zero);
         }
     } else {
-        const double* f = a.f + (long long)b * N * N * N;
+        const double* f = a.f + (long long)b * NG * NG * NG;
 #pragma unroll
         for (int s = 0; s < S; ++s) {
             T va = zero, vb = zero;
             if (s < S / 2 && on) {
-                const long long xa = (la + p) * N + t + TH * s, xb = (lb + p) * N + t + TH * s;
-                if (a.flags[xa] & 1) va = (T)(a.scale * f[swap_axes(xa, a.f_swap, N)]);
-                if (two && (a.flags[xb] & 1)) vb = (T)(a.scale * f[swap_axes(xb, a.f_swap, N)]);
+                const long long xa = (la + p) * NG + a.w2 + t + TH * s, xb = (lb + p) * NG + a.w2 + t + TH * s;
+                if (a.flags[xa] & 1) va = (T)(a.scale * f[swap_axes(xa, a.f_swap, NG)]);
+                if (two && (a.flags[xb] & 1)) vb = (T)(a.scale * f[swap_axes(xb, a.f_swap, NG)]);
             }
             v[s] = cmake<C>(va + vb, va - vb);
         }
@@ -248,13 +252,15 @@ __global__ void __launch_bounds__(EoGeo<T, L>::KT) k_eo_inv(ConvArgs<T> a, int n
     xch_sync<TH <= 32>();
     PL::template inv<true>(v, xch, p * G::XS, 1, t, a.tw);
     if (p < cnt) {
-        typename OutOf<T>::type* out = a.v + (long long)b * N * N * N;
-        const long long la = (long long)pi * N + q0 + j0 + p, lb = (long long)pj * N + q0 + j0 + p;
+        const int NG = a.N;
+        typename OutOf<T>::type* out = a.v + (long long)b * NG * NG * NG + a.w2;
+        const long long la = (long long)(pi + a.w0) * NG + q0 + j0 + a.w1 + p;
+        const long long lb = (long long)(pj + a.w0) * NG + q0 + j0 + a.w1 + p;
 #pragma unroll
         for (int s = 0; s < S / 2; ++s) {
             const int x = t + TH * s;
-            out[la * N + x] = to_out(dir_half(v[s].x + v[s].y));
-            if (two) out[lb * N + x] = to_out(dir_half(v[s].x - v[s].y));
+            out[la * NG + x] = to_out(dir_half(v[s].x + v[s].y));
+            if (two) out[lb * NG + x] = to_out(dir_half(v[s].x - v[s].y));
         }
     }
 }
@@ -560,10 +566,21 @@ void eo_configure() {
 //     623, 82 1117 / 996, 102 1231 / 1398
 // and at N <= 64 it is the faster one for every plane count (float32 N = 64:
 // 16 planes 60.9 / 54.9, 60 planes 63.8 / 63.5 with the call around it).
+// On windows, against the five passes on the same window:
+//   float32 96 nodes, one: 44 planes 48.6 / 34.7, 82 57.2 / 49.5, 96 59.6 / 57.5;
+//     32: 44 planes 491 / 249, 96 859 / 854
+//   float32 192 nodes, one: 82 planes 122 / 106, 108 187 / 159, 134 208 / 248
+//   double-float 192 nodes, operator, one: 82 planes 748 / 573, 96 772 / 690; 96
+//     nodes up to 64 planes (beyond, nine row blocks leave warps idle)
+//   float64: the passes with the direct i pass (96 nodes 44 planes 299 / 266,
+//     192 nodes 82 planes 2073 / 1945; the FP64 pipe bounds both).
 template <typename T, int L>
 constexpr int eo_limit() {
     if constexpr (L == 512) return 144;
-    else if constexpr (L == 256) return sizeof(T) == 4 ? 104 : (std::is_same<T, dsf>::value ? 72 : 86);
+    else if constexpr (L % 3 == 0 && L >= 192 && std::is_same<T, double>::value) return 0;
+    else if constexpr (L == 192 && std::is_same<T, dsf>::value) return 64;
+    else if constexpr (L == 384) return sizeof(T) == 4 ? 116 : 96;
+    else if constexpr (L >= 192) return sizeof(T) == 4 ? 104 : (std::is_same<T, dsf>::value ? 72 : 86);
     else return L / 2;
 }
 
@@ -580,7 +597,7 @@ int eo_form(const ConvArgs<T>& a, EoShape& sh) {
     if (planes > eo_limit<T, L>()) return 0;
     if constexpr (EoUse<T, L>::whole) {
         sh = eo_shape<T, L, false>(planes);
-        if (sh.w > 0 && !(L == 512 && sh.big)) return 1;
+        if (sh.w > 0 && !(L >= 384 && sh.big)) return 1;
     }
     if constexpr (EoUse<T, L>::split) {
         sh = eo_shape<T, L, true>(planes);

@@ -27,6 +27,14 @@ template <int V> struct PlanOf<dsf, 256, V> { using type = Plan3_256; };
 template <int V> struct PlanOf<double, 512, V> { using type = Plan3_512; };
 template <int V> struct PlanOf<dsf, 512, V> { using type = Plan3_512; };
 template <> struct PlanOf<float, 512, 1> { using type = Plan3_512; };
+// the windows of 3 2^p nodes
+template <typename T, int L> struct PlanWin;
+template <typename T> struct PlanWin<T, 96> { using type = PlanQ<12, 4, 2>; };
+template <typename T> struct PlanWin<T, 192> { using type = PlanQ<12, 4, 4>; };
+template <typename T> struct PlanWin<T, 384> { using type = PlanQ<12, 8, 4>; };
+template <> struct PlanWin<float, 384> { using type = PlanQ<24, 4, 4>; };
+template <typename T, int V> struct PlanOf<T, 192, V> { using type = typename PlanWin<T, 192>::type; };
+template <typename T, int V> struct PlanOf<T, 384, V> { using type = typename PlanWin<T, 384>::type; };
 
 template <typename T, int L> struct HasAlt {
     static constexpr bool value =
@@ -37,19 +45,20 @@ template <typename T, int L> struct HasAlt {
 template <typename T, int L, int V = 0> struct Geo {
     using C = cplx_t<T>;
     using PL = typename PlanOf<T, L, V>::type;
-    static constexpr bool THREE = PL::TH * PL::S == L && PL::TH > PL::S;
+    static constexpr bool Q3 = L % 3 == 0;   // window lengths
+    static constexpr bool THREE = !Q3 && PL::TH * PL::S == L && PL::TH > PL::S;
     static constexpr int TH = PL::TH, S = PL::S;   // threads per line, values per thread
     // column passes: W columns per CTA, TH threads per column (three-level:
     // 64-byte row segments at 64 threads per line, 128-byte ones at 32, so
     // that a CTA has 256 threads for the 16-byte types)
     static constexpr int WB = 65536 / (L * (int)sizeof(C));
     static constexpr int W0 = THREE ? (128 / (int)sizeof(C) / 2) * (64 / TH) : (WB > 32 ? 32 : (WB < 8 ? 8 : WB));
-    static constexpr int W = (V == 1 && !THREE && HasAlt<T, L>::value) ? W0 / 2 : W0;
+    static constexpr int W = Q3 ? (WB >= 16 && TH * 16 <= 256 ? 16 : 8) : (V == 1 && !THREE && HasAlt<T, L>::value) ? W0 / 2 : W0;
     static constexpr int CT = W * TH;
     static constexpr int XL = PL::XLEN;            // exchange positions per column
     // line passes (k): P line pairs per CTA, TH threads per pair
     static constexpr int PB = 65536 / (L * (int)sizeof(C));
-    static constexpr int P = THREE ? 256 / TH : ((256 / TH) < PB ? (256 / TH) : (PB < 4 ? 4 : PB));
+    static constexpr int P = Q3 ? (sizeof(C) == 16 ? 8 : 16) : THREE ? 256 / TH : ((256 / TH) < PB ? (256 / TH) : (PB < 4 ? 4 : PB));
     static constexpr int KT = P * TH;
     static constexpr int XS = PL::XS;              // exchange stride per pair (odd)
     // stride of a pair's source lines (2N values) in the forward k pass:
@@ -62,7 +71,9 @@ template <typename T, int L, int V = 0> struct Geo {
     // otherwise takes 123 registers, two CTAs per SM), no constraint
     // otherwise
     static constexpr bool CAP3 = THREE || (V == 1 && std::is_same<T, float>::value && L == 256);
-    static constexpr int MINB = CAP3 ? 3 : 1;
+    // (window lengths: 12 values per thread at three CTAs per SM, 24 at two in
+    // float32)
+    static constexpr int MINB = CAP3 || (Q3 && S == 12) ? 3 : (Q3 ? 2 : 1);
     // per pass, where it differs: the three-level i pass at L = 256
     // (spectral product and two transforms) fits 128 registers without
     // spilling at two CTAs per SM and runs ~3% faster so than with the
@@ -77,6 +88,7 @@ template <typename T, int L, int V = 0> struct Geo {
                                (THREE && (L == 256 || (L == 512 && sizeof(C) == 16)));
     static constexpr int minb_col(int mode) {
         if (THREE && L == 256 && mode == 1) return 2;
+        if (Q3 && sizeof(C) == 16 && mode == 1) return 2;
         if (THREE && L == 512 && mode == 1) return MINB;
         return (F4 && (mode != 2 || THREE)) ? 4 : MINB;
     }
@@ -180,8 +192,8 @@ void launch_pdl(K kernel, dim3 grid, int threads, size_t smem, cudaStream_t st, 
 // of all 2N frequencies (not for the 16-byte elements at L = 512, whose rows
 // take 8 KB each), and rows split into the even and odd frequencies.
 template <typename T, int L> struct EoUse {
-    static constexpr bool whole = L <= 256 || std::is_same<T, float>::value;
-    static constexpr bool split = L >= 128;
+    static constexpr bool whole = L <= 256 || (L == 512 && std::is_same<T, float>::value);
+    static constexpr bool split = (L >= 128 && L % 3 != 0) || L == 384;
 };
 
 // ------------------------------------------------ packed Nyquist column
@@ -224,6 +236,9 @@ __device__ __forceinline__ C line_spectrum(const C* row, int k, int N) {
     return cconj(row[2 * N - k]);
 }
 
+// L - k, the mirror image of frequency k of a transform of length L
+__device__ __forceinline__ int mirror(int k, int L) { return k == 0 ? 0 : L - k; }
+
 // slot k of column 0 after the forward j transform, from Z(k) and Z(2N - k)
 template <typename C>
 __device__ __forceinline__ C slot_split(C zk, C zr, int k, int N) {
@@ -249,7 +264,7 @@ __device__ __forceinline__ void split_column0(C* v, C* xch, int c, int t) {
 #pragma unroll
         for (int s = 0; s < PL::S; ++s) {
             const int k = PL::kidx(t, s);
-            v[s] = slot_split(v[s], xch[(L - k) & (L - 1)], k, L / 2);
+            v[s] = slot_split(v[s], xch[mirror(k, L)], k, L / 2);
         }
     }
     __syncthreads();
@@ -305,12 +320,22 @@ template <typename T, int L> struct CPlaneGeo {
 //             planes 86 / 86
 //   float64:  N = 256 122 planes 6887 / 8515; N = 128 82 planes 1057 / 1117,
 //             102 planes 1435 / 1231; N = 64 54 planes 214 / 229
-// (128 planes is also what the shared memory of the 8-byte types holds).
+// (128 planes is also what the shared memory of the 8-byte types holds). On the
+// windows of 96 and 192 nodes, whose FFT i pass is shorter, the i pass alone:
+//   float64:  192 nodes 82 planes 1137 / 2780; 96 nodes 58 planes 145 / 328
+//   double-float: 192 nodes 44 planes 116 / 522; 96 nodes 44 planes 34 / 61
+//   float32:  192 nodes 44 planes 29 / 101
 template <typename T>
 inline int direct_i_limit(int N) {
-    if constexpr (std::is_same<T, float>::value) return N >= 256 ? 132 : (N >= 128 ? 68 : 0);
-    else if constexpr (std::is_same<T, dsf>::value) return N >= 256 ? 104 : (N >= 128 ? 70 : (N >= 64 ? 44 : 0));
-    else return N >= 256 ? 128 : (N >= 128 ? 84 : (N >= 64 ? 56 : 0));
+    const bool f32 = std::is_same<T, float>::value, ds = std::is_same<T, dsf>::value;
+    switch (N) {
+        case 256: return f32 ? 132 : (ds ? 104 : 128);
+        case 192: return f32 ? 80 : (ds ? 90 : 124);
+        case 128: return f32 ? 68 : (ds ? 70 : 84);
+        case 96: return f32 ? 0 : (ds ? 56 : 84);
+        case 64: return f32 ? 0 : (ds ? 44 : 56);
+        default: return 0;
+    }
 }
 
 }  // namespace bae

@@ -70,12 +70,14 @@ __device__ __forceinline__ void kpass_fwd_tile(const ConvArgs<T>& a, int bx, int
     const long long np = a.npairs();
     const bool active = gp0 + p < np;
     const long long la = a.pair_line(gp0 + p), lb = la + 1;
+    const int NG = a.N;                                  // the grid's pitch
+    const long long na = (long long)a.grid_line(la) * NG + a.w2, nb = na + NG;   // first nodes of the two lines
     T* r = rho + p * G::RS;
 
     C v[S];
     if (a.mode == SRC_DENSITY) {
         for (int k = t; k < 2 * N; k += TH)
-            r[k] = active ? volume_or_zero(a, b, (k < N ? la : lb) * N + (k < N ? k : k - N)) : (T)0;
+            r[k] = active ? volume_or_zero(a, b, k < N ? na + k : nb + k - N) : (T)0;
         __syncthreads();
         {
             // the sources of the CTA's lines are one contiguous range of the
@@ -86,7 +88,7 @@ __device__ __forceinline__ void kpass_fwd_tile(const ConvArgs<T>& a, int bx, int
             // density) runs once, not once per line
             const long long gp1 = min(gp0 + (long long)G::P, np);
             if (gp0 < gp1) {
-                const long long l0 = a.pair_line(gp0), l1 = a.pair_line(gp1 - 1) + 2;
+                const long long l0 = a.grid_line(a.pair_line(gp0)), l1 = a.grid_line(a.pair_line(gp1 - 1)) + 2;
                 const double* q =
                     a.q + (long long)b * a.q_stride + (a.q_row ? (long long)a.q_row[b] * a.q_row_stride : 0);
                 const float* q32 = a.q32 ? a.q32 + (long long)b * a.q32_stride : nullptr;
@@ -94,11 +96,11 @@ __device__ __forceinline__ void kpass_fwd_tile(const ConvArgs<T>& a, int bx, int
                 const int npq = a.pairs_per_plane(), jlo = a.line_lo(), jhi = a.line_hi();
                 for (int s = s0 + (int)threadIdx.x; s < s1; s += (int)blockDim.x) {
                     const int lin = a.rec.src_lin[s];
-                    const int line = lin / N, ip = line / N, jl = line % N;
+                    const int line = lin / NG, ip = line / NG - a.w0, jl = line % NG - a.w1;
                     // pair within the CTA, half of the pair
                     const long long loc = (long long)(ip - a.plane_lo()) * npq + (jl - jlo) / 2 - gp0;
                     if (jl >= jlo && jl < jhi && loc >= 0 && loc < G::P)
-                        rho[loc * G::RS + (jl & 1) * N + (lin % N)] = source_value<T>(a.rec, s, q, q32);
+                        rho[loc * G::RS + ((jl - jlo) & 1) * N + (lin % NG - a.w2)] = source_value<T>(a.rec, s, q, q32);
                 }
             }
         }
@@ -109,7 +111,7 @@ __device__ __forceinline__ void kpass_fwd_tile(const ConvArgs<T>& a, int bx, int
             v[m] = (m < S / 2) ? cmake<C>(r[n], r[N + n]) : cmake<C>((T)0, (T)0);
         }
     } else {
-        const double* f = a.f + (long long)b * N * N * N;
+        const double* f = a.f + (long long)b * NG * NG * NG;
 #pragma unroll
         for (int m = 0; m < S; ++m) {
             const int n = t + TH * m;
@@ -117,9 +119,9 @@ __device__ __forceinline__ void kpass_fwd_tile(const ConvArgs<T>& a, int bx, int
             // the sample read: n in the lower half; 2N - n mirrored (BOX)
             const int nn = m < S / 2 ? n : ((BOX && n > N) ? 2 * N - n : -1);
             if (active && nn >= 0) {
-                const long long xa = la * N + nn, xb = lb * N + nn;
-                va = (a.flags[xa] & 1) ? (T)(a.scale * f[swap_axes(xa, a.f_swap, N)]) : (T)0;
-                vb = (a.flags[xb] & 1) ? (T)(a.scale * f[swap_axes(xb, a.f_swap, N)]) : (T)0;
+                const long long xa = na + nn, xb = nb + nn;
+                va = (a.flags[xa] & 1) ? (T)(a.scale * f[swap_axes(xa, a.f_swap, NG)]) : (T)0;
+                vb = (a.flags[xb] & 1) ? (T)(a.scale * f[swap_axes(xb, a.f_swap, NG)]) : (T)0;
                 if (m >= S / 2) {
                     va = -va;
                     vb = -vb;
@@ -210,7 +212,7 @@ __device__ __forceinline__ void colpass_tile(const ConvArgs<T>& a, int bx, int b
         for (int s = 0; s < S; ++s) {
             const int k = PL::kidx(t, s);
             C x = ok ? in[k * stride] : zero;
-            if (col0 && c == 0) x = slot_merge(x, in[((L - k) & (L - 1)) * stride], k, N);
+            if (col0 && c == 0) x = slot_merge(x, in[mirror(k, L) * stride], k, N);
             v[s] = x;
         }
         PL::inv(v, xch, c, W, t, a.tw);
@@ -261,7 +263,7 @@ __device__ __forceinline__ void colpass_tile(const ConvArgs<T>& a, int bx, int b
                     const int ii = k <= N ? k : L - k;
                     const T g0 = g[(long long)ii * N1 * N1], gn = g[(long long)ii * N1 * N1 + N];
                     // (g0 + gN) y(p) / 2 + (g0 - gN) conj y(-p) / 2
-                    const C yr = cconj(xch[(L - k) & (L - 1)]);
+                    const C yr = cconj(xch[mirror(k, L)]);
                     const C y = v[s];
                     const T sp = (g0 + gn) * half, sm = (g0 - gn) * half;
                     v[s] = cmake<C>(y.x * sp + yr.x * sm, y.y * sp + yr.y * sm);
@@ -360,13 +362,15 @@ __device__ __forceinline__ void kpass_inv_tile(const ConvArgs<T>& a, int bx, int
     }
     PL::inv(v, xch, p * G::XS, 1, t, a.tw);
     if (active) {
-        typename OutOf<T>::type* out = a.v + (long long)b * N * N * N;
+        const int NG = a.N;
+        const long long na = (long long)a.grid_line(la) * NG + a.w2, nb = na + NG;
+        typename OutOf<T>::type* out = a.v + (long long)b * NG * NG * NG;
 #pragma unroll
         for (int m = 0; m < S; ++m) {
             const int n = t + TH * m;
             if (m < S / 2) {
-                out[la * N + n] = to_out(v[m].x);
-                out[lb * N + n] = to_out(v[m].y);
+                out[na + n] = to_out(v[m].x);
+                out[nb + n] = to_out(v[m].y);
             }
         }
     }
@@ -585,6 +589,26 @@ __global__ void __launch_bounds__(512) k_plane_inv(ConvArgs<T> a) {
 }
 
 template <typename T, int L>
+void configure_passes() {
+    using C = cplx_t<T>;
+    using G = Geo<T, L>;
+    const size_t smem_k = (size_t)G::P * G::XS * sizeof(C) + (size_t)G::P * G::RS * sizeof(T);
+    const size_t smem_c = (size_t)G::XL * G::W * sizeof(C);
+    static const bool configured = [&]() {
+        auto set = [](auto k, size_t smem) {
+            BAE_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        };
+        set(k_kpass_fwd<T, L>, smem_k);
+        set(k_kpass_inv<T, L>, smem_k);
+        set(k_colpass<T, L, COL_FWD_J>, smem_c);
+        set(k_colpass<T, L, COL_CONV_I>, smem_c);
+        set(k_colpass<T, L, COL_INV_J>, smem_c);
+        return true;
+    }();
+    (void)configured;
+}
+
+template <typename T, int L>
 void configure_conv() {
     using C = cplx_t<T>;
     using G = Geo<T, L>;
@@ -593,11 +617,7 @@ void configure_conv() {
     const size_t smem_c = (size_t)G::XL * G::W * sizeof(C);
     // once per instantiation (thread-safe static initialisation)
     static const bool configured = [&]() {
-        BAE_CUDA(cudaFuncSetAttribute(k_kpass_fwd<T, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_k));
-        BAE_CUDA(cudaFuncSetAttribute(k_kpass_inv<T, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_k));
-        BAE_CUDA(cudaFuncSetAttribute(k_colpass<T, L, COL_FWD_J>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c));
-        BAE_CUDA(cudaFuncSetAttribute(k_colpass<T, L, COL_CONV_I>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c));
-        BAE_CUDA(cudaFuncSetAttribute(k_colpass<T, L, COL_INV_J>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c));
+        configure_passes<T, L>();
         // the persistent instantiations of the variant-0 passes
         BAE_CUDA(cudaFuncSetAttribute(k_kpass_fwd<T, L, false, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)smem_k));
@@ -780,6 +800,19 @@ void launch_sched(const ConvArgs<T>& a, cudaStream_t st, int sched) {
 
 }  // namespace
 
+// An apply on a window of L / 2 = 3 2^p nodes: the even-odd schedule, which
+// takes every plane count up to L = 96, or the five passes.
+template <typename T, int L>
+void run_window(const ConvArgs<T>& a, cudaStream_t st) {
+    if (eo_apply<T, L>(a, st)) return;
+    if constexpr (L >= 192) {
+        configure_passes<T, L>();
+        launch_passes<T, L, 0>(a, st);
+    } else {
+        throw Error(BAE_ERR_CUDA, "internal: no schedule for this window");
+    }
+}
+
 template <typename T, int L>
 void run_conv(const ConvArgs<T>& a, cudaStream_t st) {
     configure_conv<T, L>();
@@ -844,7 +877,8 @@ void run_conv(const ConvArgs<T>& a, cudaStream_t st) {
 
 template <typename T, int L>
 void conv_configure() {
-    configure_conv<T, L>();
+    if constexpr (L % 3 != 0) configure_conv<T, L>();
+    else if constexpr (L >= 192) configure_passes<T, L>();
     eo_configure<T, L>();
 }
 

@@ -97,6 +97,9 @@ __device__ __forceinline__ dsc cadd(dsc a, dsc b) { return dsc{add_nr(a.x, b.x),
 __device__ __forceinline__ dsc csub(dsc a, dsc b) { return dsc{add_nr(a.x, -b.x), add_nr(a.y, -b.y)}; }
 __device__ __forceinline__ dsc cmul(dsc a, dsc b) { return dsc{dot2(a.x, b.x, -a.y, b.y), dot2(a.x, b.y, a.y, b.x)}; }
 __device__ __forceinline__ dsc cmulc(dsc a, dsc b) { return dsc{dot2(a.x, b.x, a.y, b.y), dot2(a.y, b.x, -a.x, b.y)}; }
+__device__ __forceinline__ dsc chalf(dsc a) {
+    return dsc{dsf(0.5f * a.x.hi, 0.5f * a.x.lo), dsf(0.5f * a.y.hi, 0.5f * a.y.lo)};
+}
 __device__ __forceinline__ dsc crot(dsc x, dsf c, dsf s) { return dsc{dot2(x.x, c, -x.y, s), dot2(x.x, s, x.y, c)}; }
 
 template <>

@@ -44,28 +44,48 @@ __host__ __device__ constexpr Root32 root32(int m) {
     return {sr, -cr};
 }
 
+// cos and sin of 2 pi m / 24, the same for the lengths with a factor of three
+__host__ __device__ constexpr Root32 root24(int m) {
+    // cos(pi j / 12), j = 0..6
+    constexpr double C[7] = {1.0, 0.96592582628906828675, 0.86602540378443864676, 0.70710678118654752440,
+                             0.5, 0.25881904510252076235, 0.0};
+    m = ((m % 24) + 24) % 24;
+    const int q = m / 6, r = m % 6;
+    const double cr = C[r], sr = C[6 - r];
+    if (q == 0) return {cr, sr};
+    if (q == 1) return {-sr, cr};
+    if (q == 2) return {-cr, -sr};
+    return {sr, -cr};
+}
+// cos and sin of 2 pi M / R, R dividing 32 or 24
+template <int R>
+__host__ __device__ constexpr Root32 root_of(int M) {
+    if constexpr (32 % R == 0) return root32(M * (32 / R));
+    else return root24(M * (24 / R));
+}
+
 // x (c + i s)
 template <typename C, typename T>
 __device__ __forceinline__ C crot(C x, T c, T s) {
     return cmake<C>(x.x * c - x.y * s, x.x * s + x.y * c);
 }
 
-// x * exp(-/+ 2 pi i M / R) with compile-time M, R | 32
+// x * exp(-/+ 2 pi i M / R) with compile-time M, R dividing 32 or 24
 template <int R, int M, bool INV, typename C>
 __device__ __forceinline__ C wmul(C x) {
     using T = decltype(x.x);
-    constexpr int m = ((M * (32 / R)) % 32 + 32) % 32;
+    constexpr int m = ((M % R) + R) % R;
     if constexpr (m == 0) return x;
-    if constexpr (m == 16) return cmake<C>(-x.x, -x.y);
-    if constexpr (m == 8) {   // forward: -i, inverse: +i
+    if constexpr (2 * m == R) return cmake<C>(-x.x, -x.y);
+    if constexpr (4 * m == R) {       // forward: -i, inverse: +i
         if constexpr (INV) return cmake<C>(-x.y, x.x);
         else return cmake<C>(x.y, -x.x);
     }
-    if constexpr (m == 24) {  // forward: +i, inverse: -i
+    if constexpr (4 * m == 3 * R) {   // forward: +i, inverse: -i
         if constexpr (INV) return cmake<C>(x.y, -x.x);
         else return cmake<C>(-x.y, x.x);
     }
-    constexpr Root32 w = root32(m);
+    constexpr Root32 w = root_of<R>(m);
     const T c = (T)w.c;
     const T s = INV ? (T)w.s : (T)-w.s;
     return crot(x, c, s);
@@ -103,13 +123,12 @@ __device__ __forceinline__ double fma_t(double a, double b, double c) { return _
 template <int R, int K, bool INV, typename C>
 __device__ __forceinline__ void bfly(const C& e, const C& o, C& lo, C& hi) {
     using T = decltype(o.x);
-    constexpr int m = ((K * (32 / R)) % 32 + 32) % 32;
-    if constexpr (!(std::is_same<T, float>::value || std::is_same<T, double>::value) || m % 8 == 0) {
+    if constexpr (!(std::is_same<T, float>::value || std::is_same<T, double>::value) || (4 * K) % R == 0) {
         const C w = wmul<R, K, INV>(o);
         lo = cadd(e, w);
         hi = csub(e, w);
     } else {
-        constexpr Root32 w = root32(m);
+        constexpr Root32 w = root_of<R>(K);
         constexpr double c = w.c, sn = INV ? w.s : -w.s;   // W = c + i sn
         T ux, uy, f;
         if constexpr (c * c >= sn * sn) {   // W = c (1 + i sn/c)
@@ -137,7 +156,32 @@ struct Bflies {
     }
 };
 
-// In-register DFT of v[0..R) in natural order, R in {2, 4, 8, 16, 32}.
+// x / 2
+template <typename C>
+__device__ __forceinline__ C chalf(C x) {
+    using T = decltype(x.x);
+    return cmake<C>(x.x * (T)0.5, x.y * (T)0.5);
+}
+
+// Three points: y0 = x0 + x1 + x2, y1, y2 = x0 - (x1 + x2) / 2 -/+ i (sqrt 3 /
+// 2) (x1 - x2) (forward). NZ: how many of the inputs are nonzero.
+template <bool INV, int NZ, typename C>
+__device__ __forceinline__ void rdft3(C* v) {
+    using T = decltype(v[0].x);
+    if constexpr (NZ == 1) {
+        v[1] = v[2] = v[0];
+        return;
+    }
+    const C t = NZ == 2 ? v[1] : cadd(v[1], v[2]);
+    const C d = cscale(NZ == 2 ? v[1] : csub(v[1], v[2]), (T)0.86602540378443864676);
+    const C m = csub(v[0], chalf(t));
+    const C e = INV ? cmake<C>(-d.y, d.x) : cmake<C>(d.y, -d.x);   // +i d, -i d
+    v[0] = cadd(v[0], t);
+    v[1] = cadd(m, e);
+    v[2] = csub(m, e);
+}
+
+// In-register DFT of v[0..R) in natural order, R = 2^p <= 32 or 3 2^p <= 24.
 template <int R, bool INV, typename C>
 __device__ __forceinline__ void rdft(C* v);
 
@@ -145,6 +189,8 @@ template <int R, bool INV, typename C>
 __device__ __forceinline__ void rdft(C* v) {
     if constexpr (R == 2) {
         rdft2<INV>(v[0], v[1]);
+    } else if constexpr (R == 3) {
+        rdft3<INV, 3>(v);
     } else if constexpr (R == 4) {
         rdft4<INV>(v[0], v[1], v[2], v[3]);
     } else {
@@ -175,6 +221,10 @@ __device__ __forceinline__ void rdft_zhi(C* v) {
         v[2] = csub(x0, x1);
         v[1] = cadd(x0, t3);
         v[3] = csub(x0, t3);
+    } else if constexpr (R == 6) {   // v[0..3) nonzero
+        C e[3] = {v[0], v[2], v[2]}, o[3] = {v[1], v[1], v[1]};
+        rdft3<INV, 2>(e);
+        Bflies<R, INV, C, 0>::run(e, o, v);
     } else {
         C e[R / 2], o[R / 2];   // both halves have a zero upper half again
 #pragma unroll
@@ -454,6 +504,94 @@ struct Plan3_256 {
 #pragma unroll
         for (int j3 = 1; j3 < 8; ++j3) v[j3] = cmulc(v[j3], ldg_c(tw + t * j3));
         rdft<8, true>(v);                                // v[m] = x[t + 32 m]
+    }
+};
+
+// Three levels for the lengths 3 2^p: L = RA x RB x RC, TH = RB RC threads per
+// line (a power of two, within a warp), RA = 12 or 24 values each (12 x 8 x 4 for
+// 16-byte elements at L = 384: with 24 values they take 255 registers). With n = t +
+// TH m, t = t1 + RC t2, k = k3 + RA k2 + RA RB k1:
+//   X[k] = sum_t1 W_RC^{t1 k1} W_TH^{t1 k2} sum_t2 W_RB^{t2 k2}
+//          [ W_L^{t k3} sum_m W_RA^{m k3} x[t + TH m] ]
+// stage A: thread t, DFT over m; exchange; stage B: RA / RB transforms (k3, t1)
+// per thread over t2, in place in the exchange area; stage C: RA / RC
+// transforms (k3, k2) per thread over t1. Rows of TH values are PITCH = TH + RC
+// + 1 apart, so that the 16 lanes of a half warp read distinct 8-byte banks in
+// stage C (rows k3 = lane mod RA: 21 k3 mod 16 for TH = 16) and nearly so in B.
+template <int RA, int RB, int RC>
+struct PlanQ {
+    static constexpr int TH = RB * RC, S = RA, L = RA * TH;
+    static constexpr int PITCH = TH + RC + 1, XLEN = RA * PITCH, XS = XLEN | 1;
+    static constexpr int QB = (RA + RB - 1) / RB;   // stage B transforms per thread (the last round may be partial)
+    static_assert(RA % RC == 0 && TH <= 32, "a line in a warp, whole stage C transforms per thread");
+    // slot s = q RC + k1 of thread t holds X[t + TH q + RA RB k1]
+    __host__ __device__ static constexpr int kidx(int t, int s) { return t + TH * (s / RC) + RA * RB * (s % RC); }
+
+    template <bool ZHI, bool WARP = false, typename C>
+    __device__ __forceinline__ static void fwd(C* v, C* xch, int base, int es, int t, const C* __restrict__ tw) {
+        if constexpr (ZHI) rdft_zhi<RA, false>(v);
+        else rdft<RA, false>(v);
+#pragma unroll
+        for (int k3 = 1; k3 < RA; ++k3) v[k3] = cmul(v[k3], ldg_c(WARP && TH <= 16 ? tw + L + k3 * TH + t : tw + t * k3));
+#pragma unroll
+        for (int k3 = 0; k3 < RA; ++k3) xch[base + (k3 * PITCH + t) * es] = v[k3];
+        xch_sync<WARP>();
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
+            const int i = t + TH * q, k3 = i / RC, t1 = i % RC;
+            if (RA % RB != 0 && k3 >= RA) continue;
+            C* x = xch + base + (k3 * PITCH + t1) * es;
+            C w[RB];
+#pragma unroll
+            for (int t2 = 0; t2 < RB; ++t2) w[t2] = x[t2 * RC * es];
+            rdft<RB, false>(w);
+            x[0] = w[0];
+#pragma unroll
+            for (int k2 = 1; k2 < RB; ++k2) x[k2 * RC * es] = cmul(w[k2], ldg_c(tw + RA * t1 * k2));
+        }
+        xch_sync<WARP>();
+#pragma unroll
+        for (int q = 0; q < RA / RC; ++q) {
+            const int i = t + TH * q, k3 = i % RA, k2 = i / RA;
+            const C* x = xch + base + (k3 * PITCH + k2 * RC) * es;
+#pragma unroll
+            for (int t1 = 0; t1 < RC; ++t1) v[q * RC + t1] = x[t1 * es];
+            rdft<RC, false>(v + q * RC);
+        }
+        xch_sync<WARP>();
+    }
+
+    template <bool WARP = false, typename C>
+    __device__ __forceinline__ static void inv(C* v, C* xch, int base, int es, int t, const C* __restrict__ tw) {
+#pragma unroll
+        for (int q = 0; q < RA / RC; ++q) {
+            const int i = t + TH * q, k3 = i % RA, k2 = i / RA;
+            C* x = xch + base + (k3 * PITCH + k2 * RC) * es;
+            rdft<RC, true>(v + q * RC);
+#pragma unroll
+            for (int t1 = 0; t1 < RC; ++t1) x[t1 * es] = v[q * RC + t1];
+        }
+        xch_sync<WARP>();
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
+            const int i = t + TH * q, k3 = i / RC, t1 = i % RC;
+            if (RA % RB != 0 && k3 >= RA) continue;
+            C* x = xch + base + (k3 * PITCH + t1) * es;
+            C w[RB];
+            w[0] = x[0];
+#pragma unroll
+            for (int k2 = 1; k2 < RB; ++k2) w[k2] = cmulc(x[k2 * RC * es], ldg_c(tw + RA * t1 * k2));
+            rdft<RB, true>(w);
+#pragma unroll
+            for (int t2 = 0; t2 < RB; ++t2) x[t2 * RC * es] = w[t2];
+        }
+        xch_sync<WARP>();
+        v[0] = xch[base + t * es];
+#pragma unroll
+        for (int k3 = 1; k3 < RA; ++k3)
+            v[k3] = cmulc(xch[base + (k3 * PITCH + t) * es], ldg_c(WARP && TH <= 16 ? tw + L + k3 * TH + t : tw + t * k3));
+        xch_sync<WARP>();
+        rdft<RA, true>(v);   // v[m] = x[t + TH m]
     }
 };
 

@@ -392,9 +392,9 @@ __global__ void k_twiddles(int L, double2* tw64, float2* tw32) {
     }
 }
 
-// first thread count of the two-level split of a transform of length L
-// (Factors<L>::R1)
-__host__ __device__ inline int level_one(int L) { return L <= 32 ? 4 : (L <= 128 ? 8 : 16); }
+// threads per line of the plans that read the products table of a transform
+// of length L (Factors<L>::R1; PlanQ with at most 16 threads)
+__host__ __device__ inline int level_one(int L) { return L <= 48 ? 4 : (L <= 128 ? 8 : 16); }
 
 // out[k2 R1 + n1] = exp(-2 pi i n1 k2 / L), n1 < R1, k2 < L / R1
 __global__ void k_twiddle_products(int L, int R1, double2* tw64, float2* tw32) {

@@ -65,7 +65,7 @@ void apply_into(const ProblemView& pv, const double* q, double* v, unsigned char
                         " bytes of scratch; the static scratch holds " + std::to_string(kNoAllocScratchBytes) +
                         " (float32: N <= 64, float64: N <= 32)");
     ConvArgs<T> a;
-    a.N = pv.N;
+    a.N = a.nt = pv.N;
     a.nbatch = 1;
     a.mode = SRC_DENSITY;
     a.q = q;

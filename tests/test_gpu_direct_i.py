@@ -6,6 +6,8 @@ thinnest the geometry allows to the most planes the direct sum takes, odd and
 even plane counts, off-centre, both layers; float64 and double-float to 1e-12
 and float32 to 2e-6 of the largest potential, the bounds of the oracle
 comparisons of the same applies."""
+import contextlib
+
 import numpy as np
 import pytest
 
@@ -49,14 +51,13 @@ def test_direct_sum_matches_fft(ctx, N, half, z0, layer, precision, schedule):
     import torch
     from paper_2502_05507_gb300 import Problem, set_conv_schedule
     P = slab(N, half, z0, 5.0)
-    prob = Problem(ctx, torch.from_numpy(P.phi).cuda(), P.grid.h, P.grid.origin, P.kappa2, layer)
-    ax, lo, hi = prob.conv_planes()
-    cl = prob.classification()
-    q = torch.from_numpy(W.random_density(prob.n_unknowns, seed=61)).cuda()
-    set_conv_schedule("passes")
-    v = prob.potential_apply(q, "fp64").cpu().numpy().reshape(-1)
-    ref = cl["t"] * v[cl["gm"]] + (1.0 - cl["t"]) * v[cl["partner"]]
-    set_conv_schedule(schedule)
-    Aq = prob.boundary_apply(q, precision).cpu().numpy()
-    assert np.max(np.abs(Aq - ref)) <= TOL[precision] * np.max(np.abs(v)), (ax, lo, hi)
-    prob.close()
+    with contextlib.closing(Problem(ctx, torch.from_numpy(P.phi).cuda(), P.grid.h, P.grid.origin, P.kappa2, layer)) as prob:
+        ax, lo, hi = prob.conv_planes()
+        cl = prob.classification()
+        q = torch.from_numpy(W.random_density(prob.n_unknowns, seed=61)).cuda()
+        set_conv_schedule("passes")
+        v = prob.potential_apply(q, "fp64").cpu().numpy().reshape(-1)
+        ref = cl["t"] * v[cl["gm"]] + (1.0 - cl["t"]) * v[cl["partner"]]
+        set_conv_schedule(schedule)
+        Aq = prob.boundary_apply(q, precision).cpu().numpy()
+        assert np.max(np.abs(Aq - ref)) <= TOL[precision] * np.max(np.abs(v)), (ax, lo, hi)
