@@ -23,7 +23,8 @@
 // Measured at N = 128, 32 planes, 64 right-hand sides (five passes with the
 // direct i pass / these): float32 789 / 468 us per apply (the middle pass 317:
 // 70% of the issue slots, a fifth of HBM), double-float 3.21 / 2.77 ms (the
-// float32 pipes).
+// float32 pipes). On the window of 96 nodes that torus fits: float32 357 us (the
+// middle pass 230), double-float 1.83 ms.
 // Rows of A hold the lines [q0, q1) only, and column 0 packs the real kk = 0
 // and kk = N spectra as in the five passes (conv_geo.cuh).
 #pragma once
@@ -38,8 +39,9 @@ template <typename T, int L> struct EoPlan { using type = Plan2<L>; };
 template <> struct EoPlan<double, 256> { using type = Plan3_256; };
 template <> struct EoPlan<dsf, 256> { using type = Plan3_256; };
 template <typename T> struct EoPlan<T, 96> : PlanWin<T, 96> {};
-template <typename T> struct EoPlan<T, 192> : PlanWin<T, 192> {};
+template <typename T> struct EoPlan<T, 192> { using type = PlanL<12>; };
 template <typename T> struct EoPlan<T, 384> : PlanWin<T, 384> {};
+template <> struct EoPlan<float, 384> { using type = PlanL<24>; };
 template <> struct EoPlan<double, 512> { using type = Plan3_512; };
 template <> struct EoPlan<dsf, 512> { using type = Plan3_512; };
 
@@ -48,7 +50,11 @@ template <> struct EoPlan<dsf, 512> { using type = Plan3_512; };
 template <typename T, int L> struct EoGeo {
     using C = cplx_t<T>;
     using PL = typename EoPlan<T, L>::type;
-    static constexpr int TH = PL::TH, S = PL::S, XS = PL::XS;
+    static constexpr int TH = PL::TH, S = PL::S;
+    // lines of the k passes XS values apart: 2 mod 16 (8-byte values) or odd, so
+    // that the transposed accesses (lanes: 8 lines of 2 or 1 frequencies) touch
+    // distinct banks
+    static constexpr int XS = sizeof(C) == 8 ? (PL::XS + 12) / 16 * 16 + 2 : PL::XS;
     static constexpr int P = 8, KT = P * TH;
     static constexpr int RS = L + (sizeof(T) == 4 && TH < 32 ? TH : 0);
     static constexpr size_t SMEM_KF = (size_t)P * XS * sizeof(C) + (size_t)P * RS * sizeof(T);

@@ -595,4 +595,85 @@ struct PlanQ {
     }
 };
 
+// PlanQ<RA, 4, 4> for lines with private areas (line passes only: the exchange
+// has unit stride). Rows of 16 values, the value of column x in row k3 at
+// 16 k3 + (x ^ 5 (k3 mod 4)), and stage C's transforms dealt to the threads as k2 =
+// t mod 4, k3 = t / 4 + 4 q: every access of a half warp (one line) then touches
+// 16 distinct 8-byte banks in all three stages, where the padded rows of PlanQ
+// take two passes in stages B and C, and a line takes L values instead of 21 RA
+// (the float32 even-odd kernels at L = 192, 64 right-hand sides: 80.7 + 258 + 66.3
+// to 68.9 + 230 + 58.0 us).
+template <int RA>
+struct PlanL {
+    static constexpr int TH = 16, S = RA, L = 16 * RA, XLEN = L, XS = L + 1;
+    static_assert(RA % 4 == 0, "four-point transforms");
+    // slot s = 4 q + k1 of thread t holds X[t / 4 + 4 q + RA (t mod 4) + 4 RA k1]
+    __host__ __device__ static constexpr int kidx(int t, int s) { return t / 4 + 4 * (s / 4) + RA * (t % 4) + 4 * RA * (s % 4); }
+    __device__ __forceinline__ static int pos(int k3, int x) { return 16 * k3 + (x ^ (5 * (k3 & 3))); }
+
+    template <bool ZHI, bool WARP, typename C>
+    __device__ __forceinline__ static void fwd(C* v, C* xch, int base, int, int t, const C* __restrict__ tw) {
+        C* x = xch + base;
+        if constexpr (ZHI) rdft_zhi<RA, false>(v);
+        else rdft<RA, false>(v);
+#pragma unroll
+        for (int k3 = 1; k3 < RA; ++k3) v[k3] = cmul(v[k3], ldg_c(tw + L + k3 * 16 + t));
+#pragma unroll
+        for (int k3 = 0; k3 < RA; ++k3) x[pos(k3, t)] = v[k3];
+        xch_sync<WARP>();
+        const int t1 = t & 3, th = t >> 2;
+#pragma unroll
+        for (int q = 0; q < RA / 4; ++q) {   // row k3 = th + 4 q, so k3 mod 4 = th
+            C* r = x + 16 * (th + 4 * q);
+            C w[4];
+#pragma unroll
+            for (int t2 = 0; t2 < 4; ++t2) w[t2] = r[(t1 + 4 * t2) ^ (5 * th)];
+            rdft4<false>(w[0], w[1], w[2], w[3]);
+#pragma unroll
+            for (int k2 = 0; k2 < 4; ++k2)
+                r[(t1 + 4 * k2) ^ (5 * th)] = k2 == 0 ? w[0] : cmul(w[k2], ldg_c(tw + RA * t1 * k2));
+        }
+        xch_sync<WARP>();
+#pragma unroll
+        for (int q = 0; q < RA / 4; ++q) {
+            const C* r = x + 16 * (th + 4 * q);
+#pragma unroll
+            for (int u1 = 0; u1 < 4; ++u1) v[4 * q + u1] = r[(u1 + 4 * t1) ^ (5 * th)];   // k2 = t mod 4
+            rdft4<false>(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        }
+        xch_sync<WARP>();
+    }
+
+    template <bool WARP, typename C>
+    __device__ __forceinline__ static void inv(C* v, C* xch, int base, int, int t, const C* __restrict__ tw) {
+        C* x = xch + base;
+        const int t1 = t & 3, th = t >> 2;
+#pragma unroll
+        for (int q = 0; q < RA / 4; ++q) {
+            C* r = x + 16 * (th + 4 * q);
+            rdft4<true>(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+#pragma unroll
+            for (int u1 = 0; u1 < 4; ++u1) r[(u1 + 4 * t1) ^ (5 * th)] = v[4 * q + u1];
+        }
+        xch_sync<WARP>();
+#pragma unroll
+        for (int q = 0; q < RA / 4; ++q) {
+            C* r = x + 16 * (th + 4 * q);
+            C w[4];
+            w[0] = r[t1 ^ (5 * th)];
+#pragma unroll
+            for (int k2 = 1; k2 < 4; ++k2) w[k2] = cmulc(r[(t1 + 4 * k2) ^ (5 * th)], ldg_c(tw + RA * t1 * k2));
+            rdft4<true>(w[0], w[1], w[2], w[3]);
+#pragma unroll
+            for (int t2 = 0; t2 < 4; ++t2) r[(t1 + 4 * t2) ^ (5 * th)] = w[t2];
+        }
+        xch_sync<WARP>();
+        v[0] = x[pos(0, t)];
+#pragma unroll
+        for (int k3 = 1; k3 < RA; ++k3) v[k3] = cmulc(x[pos(k3, t)], ldg_c(tw + L + k3 * 16 + t));
+        xch_sync<WARP>();
+        rdft<RA, true>(v);   // v[m] = x[t + 16 m]
+    }
+};
+
 }  // namespace bae
