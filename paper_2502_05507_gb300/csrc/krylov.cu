@@ -206,9 +206,11 @@ __device__ __forceinline__ RowView shared_rows(const double* sV) {
 }
 
 // The update of step j on the chunk [r0, r0 + ACH): with
-// S_c = sum_{i<j} V[i] c[i] and S_b = sum_{i<j} V[i] b[i] (8 warps split the
-// rows, warp q taking rows q, q + 8, ..., four rows per loop trip so that
-// eight loads are in flight; partial sums added in warp order),
+// S_c = sum_{i<j} V[i] c[i] and S_b = sum_{i<j} V[i] b[i] (for j > 16 the 8
+// warps split the rows, warp q taking rows q, q + 8, ..., four rows per loop
+// trip so that eight loads are in flight; for fewer rows thread e + 64 g takes
+// element e of rows g, g + 4, ..., so that half as many partial sums are left to
+// add; partial sums added in order),
 //   q_j = (u_j - S_c) inv,   u_{j+1} = (w - S_b - q_j t) inv,
 // u_j read from row j of the view. q_j goes to row j of Vg and u_{j+1} to
 // row j + 1 (and its float32 copy to v32). Indices past the end of the
@@ -216,40 +218,55 @@ __device__ __forceinline__ RowView shared_rows(const double* sV) {
 __device__ __forceinline__ void chunk_next(const RowView& V, long long n, long long r0, int j, const double* s_c,
                                            const double* s_b, double t, double inv, const double* w, double* Vg,
                                            float* v32, double* s_acc) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0;
-    int i = warp;
-    for (; i + 24 < j; i += 32) {
-        const double* v0 = V.base + (long long)i * V.rs;
-        const double* v1 = v0 + 8 * V.rs;
-        const double* v2 = v0 + 16 * V.rs;
-        const double* v3 = v0 + 24 * V.rs;
-        const double x0 = v0[V.oa], y0 = v0[V.ob], x1 = v1[V.oa], y1 = v1[V.ob];
-        const double x2 = v2[V.oa], y2 = v2[V.ob], x3 = v3[V.oa], y3 = v3[V.ob];
-        a0 += x0 * s_c[i] + x1 * s_c[i + 8] + x2 * s_c[i + 16] + x3 * s_c[i + 24];
-        a1 += y0 * s_c[i] + y1 * s_c[i + 8] + y2 * s_c[i + 16] + y3 * s_c[i + 24];
-        b0 += x0 * s_b[i] + x1 * s_b[i + 8] + x2 * s_b[i + 16] + x3 * s_b[i + 24];
-        b1 += y0 * s_b[i] + y1 * s_b[i + 8] + y2 * s_b[i + 16] + y3 * s_b[i + 24];
+    const bool few = j <= 16;
+    if (few) {
+        const int e = threadIdx.x & (ACH - 1), g = threadIdx.x / ACH;
+        double pc = 0.0, pb = 0.0;
+#pragma unroll 4
+        for (int i = g; i < j; i += 4) {
+            const double x = V.at(i, e);
+            pc = __fma_rn(x, s_c[i], pc);
+            pb = __fma_rn(x, s_b[i], pb);
+        }
+        s_acc[g * ACH + e] = pc;
+        s_acc[(8 + g) * ACH + e] = pb;
+    } else {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0;
+        int i = warp;
+        for (; i + 24 < j; i += 32) {
+            const double* v0 = V.base + (long long)i * V.rs;
+            const double* v1 = v0 + 8 * V.rs;
+            const double* v2 = v0 + 16 * V.rs;
+            const double* v3 = v0 + 24 * V.rs;
+            const double x0 = v0[V.oa], y0 = v0[V.ob], x1 = v1[V.oa], y1 = v1[V.ob];
+            const double x2 = v2[V.oa], y2 = v2[V.ob], x3 = v3[V.oa], y3 = v3[V.ob];
+            a0 += x0 * s_c[i] + x1 * s_c[i + 8] + x2 * s_c[i + 16] + x3 * s_c[i + 24];
+            a1 += y0 * s_c[i] + y1 * s_c[i + 8] + y2 * s_c[i + 16] + y3 * s_c[i + 24];
+            b0 += x0 * s_b[i] + x1 * s_b[i + 8] + x2 * s_b[i + 16] + x3 * s_b[i + 24];
+            b1 += y0 * s_b[i] + y1 * s_b[i + 8] + y2 * s_b[i + 16] + y3 * s_b[i + 24];
+        }
+        for (; i < j; i += 8) {
+            const double* v = V.base + (long long)i * V.rs;
+            const double x = v[V.oa], y = v[V.ob];
+            a0 += x * s_c[i];
+            a1 += y * s_c[i];
+            b0 += x * s_b[i];
+            b1 += y * s_b[i];
+        }
+        s_acc[warp * ACH + lane] = a0;
+        s_acc[warp * ACH + lane + 32] = a1;
+        s_acc[(8 + warp) * ACH + lane] = b0;
+        s_acc[(8 + warp) * ACH + lane + 32] = b1;
     }
-    for (; i < j; i += 8) {
-        const double* v = V.base + (long long)i * V.rs;
-        const double x = v[V.oa], y = v[V.ob];
-        a0 += x * s_c[i];
-        a1 += y * s_c[i];
-        b0 += x * s_b[i];
-        b1 += y * s_b[i];
-    }
-    s_acc[warp * ACH + lane] = a0;
-    s_acc[warp * ACH + lane + 32] = a1;
-    s_acc[(8 + warp) * ACH + lane] = b0;
-    s_acc[(8 + warp) * ACH + lane + 32] = b1;
     __syncthreads();
     if (threadIdx.x < ACH) {
         const int e = threadIdx.x;
         const long long r = r0 + e;
-        double sc = 0.0, sb = 0.0;
+        double sc = s_acc[e], sb = s_acc[8 * ACH + e];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 1; q < 8; ++q) {
+            if (few && q >= 4) break;
             sc += s_acc[q * ACH + e];
             sb += s_acc[(8 + q) * ACH + e];
         }
@@ -264,52 +281,45 @@ __device__ __forceinline__ void chunk_next(const RowView& V, long long n, long l
     __syncthreads();
 }
 
+// partial dots of the chunk against rows i < cols, at most 16: part[i][c] for
+// the vector s_u (two != 0: and part2[i][c] for s_w). Warps 0-3 take u, warps
+// 4-7 w, each four rows: lane e sums the elements e and e + 32 of its rows,
+// then the four sums meet in a halving exchange (lanes 16 apart trade two sums
+// each, lanes 8 apart one, and the last eight lanes add up one), so a group of
+// four rows costs 14 float64 warp instructions. Each holds GB300's FP64 pipe
+// for 64 cycles, which is what bounds the step of many right-hand sides: with
+// lanes over (row, element group) pairs and a sum over eight warps nine rows of
+// both vectors took 110 instead of 84 of them.
+__device__ __forceinline__ void chunk_dots_few(const RowView& V, int cols, const double* s_u, const double* s_w,
+                                               bool two, double* part, double* part2, int nch, int c) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int r0 = 4 * (warp & 3);
+    if (r0 >= cols || (warp >= 4 && !two)) return;
+    const double* x = warp < 4 ? s_u : s_w;
+    const double x0 = x[lane], x1 = x[lane + 32];
+    double p[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const double* v = V.base + (long long)min(r0 + k, cols - 1) * V.rs;
+        p[k] = __fma_rn(v[V.ob], x1, v[V.oa] * x0);
+    }
+    const bool up = lane & 16, mid = lane & 8;
+    double a = (up ? p[2] : p[0]) + __shfl_xor_sync(0xffffffffu, up ? p[0] : p[2], 16);
+    double b = (up ? p[3] : p[1]) + __shfl_xor_sync(0xffffffffu, up ? p[1] : p[3], 16);
+    double t = (mid ? b : a) + __shfl_xor_sync(0xffffffffu, mid ? a : b, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    const int row = r0 + (up ? 2 : 0) + (mid ? 1 : 0);
+    if ((lane & 7) == 0 && row < cols) (warp < 4 ? part : part2)[(long long)row * nch + c] = t;
+}
+
 // partial dots of the chunk against rows i < cols: part[i][c]. Warp q sums
 // the elements [8q, 8q + 8) of 32 rows at a time (lane = row, two
 // accumulators), then warp 0 adds the eight warp partials of its row in
 // warp order: ~2 float64 warp instructions per row instead of a shuffle
-// tree per row (each float64 warp instruction occupies GB300's FP64 pipe
-// for ~64 cycles). s_red: 8 x 32 doubles of shared memory.
-// The same sums when at most 32 / G rows are used (the first Arnoldi steps
-// of a cycle): lane = (row r = lane % R, element group g = lane / R), each
-// lane sums its row over the 8 / G elements g, g + G, ... of the warp's 8,
-// and the G groups meet through the shuffle tree, so a float64 warp
-// instruction has (nearly) all lanes busy instead of one per row.
-template <int G>
-__device__ __forceinline__ void chunk_dots_grouped(const RowView& V, int cols, const double* s_w, double* part,
-                                                   int nch, int c, double* s_red) {
-    constexpr int R = 32 / G, E = 8 / G;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int r = lane % R, g = lane / R;
-    double acc = 0.0;
-    if (r < cols) {
-        double p0 = 0.0, p1 = 0.0;
-#pragma unroll
-        for (int u = 0; u < E; ++u) {
-            const int e = 8 * warp + g + G * u;
-            if (u & 1) p1 = __fma_rn(V.at(r, e), s_w[e], p1);
-            else p0 = __fma_rn(V.at(r, e), s_w[e], p0);
-        }
-        acc = E > 1 ? p0 + p1 : p0;
-    }
-#pragma unroll
-    for (int o = R; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (g == 0) s_red[warp * 32 + r] = acc;
-    __syncthreads();
-    if (warp == 0 && lane < cols) {
-        double t = s_red[lane];
-#pragma unroll
-        for (int q = 1; q < 8; ++q) t += s_red[q * 32 + lane];
-        part[(long long)lane * nch + c] = t;
-    }
-    __syncthreads();
-}
-
+// tree per row. s_red: 8 x 32 doubles of shared memory.
 __device__ __forceinline__ void chunk_dots(const RowView& V, int cols, const double* s_w, double* part, int nch,
                                            int c, double* s_red) {
-    if (cols <= 4) return chunk_dots_grouped<8>(V, cols, s_w, part, nch, c, s_red);
-    if (cols <= 8) return chunk_dots_grouped<4>(V, cols, s_w, part, nch, c, s_red);
-    if (cols <= 16) return chunk_dots_grouped<2>(V, cols, s_w, part, nch, c, s_red);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double wv[8];
 #pragma unroll
@@ -338,6 +348,18 @@ __device__ __forceinline__ void chunk_dots(const RowView& V, int cols, const dou
             part[(long long)i * nch + c] = t;
         }
         __syncthreads();
+    }
+}
+
+// the partial dots of step j's chunk: Q^T u and u.u to part, and when ran
+// Q^T w and u.w to part2
+__device__ __forceinline__ void step_dots(const RowView& V, int cols, const double* s_u, const double* s_w, bool ran,
+                                          double* part, double* part2, int nch, int c, double* s_red) {
+    if (cols <= 16) {
+        chunk_dots_few(V, cols, s_u, s_w, ran, part, part2, nch, c);
+    } else {
+        chunk_dots(V, cols, s_u, part, nch, c, s_red);
+        if (ran) chunk_dots(V, cols, s_w, part2, nch, c, s_red);
     }
 }
 
@@ -529,8 +551,7 @@ __global__ void __launch_bounds__(256) k_arn_dots(Arnoldi a) {
     __syncthreads();
     double* part = a.part + (long long)b * 2 * (m + 1) * a.nchunk;
     const RowView V = global_rows(Vb, a.n, r0);
-    chunk_dots(V, j + 1, s_u, part, a.nchunk, c, s_red8);
-    if (ran) chunk_dots(V, j + 1, s_w, part + (long long)(m + 1) * a.nchunk, a.nchunk, c, s_red8);
+    step_dots(V, j + 1, s_u, s_w, ran, part, part + (long long)(m + 1) * a.nchunk, a.nchunk, c, s_red8);
     if (last_block(a.ctr + 3 * b + 0, gridDim.x, &s_last)) {
         step_coeffs(a, b, j, ran, s_cf, s_rt);
         if (ran) publish_coeffs(a, b, j, s_cf, s_rt);
@@ -703,8 +724,7 @@ __global__ void __launch_bounds__(256, 4) k_arn_step_coop(Arnoldi a) {
         __syncthreads();
         const RowView V = SV ? shared_rows(s_V) : global_rows(Vb, a.n, r0);
         double* part = a.part + (long long)b * 2 * (m + 1) * a.nchunk;
-        chunk_dots(V, j + 1, s_u, part, a.nchunk, c, s_acc);
-        if (ran) chunk_dots(V, j + 1, s_w, part + (long long)(m + 1) * a.nchunk, a.nchunk, c, s_acc);
+        step_dots(V, j + 1, s_u, s_w, ran, part, part + (long long)(m + 1) * a.nchunk, a.nchunk, c, s_acc);
         __syncthreads();
     }
     if (!grid_barrier(a.bar, G + a.bar_extra, a.err, a.err_host, a.spin_limit)) return;   // all G CTAs
@@ -774,15 +794,19 @@ __global__ void __launch_bounds__(256, 4) k_arn_step_coop(Arnoldi a) {
         float xv[RW];
 #pragma unroll
         for (int u = 0; u < RW; ++u) xv[u] = r0 + u < a.n ? __ldcg(x + pc[u]) : 0.f;
+        // lane u keeps row u's sum: one float64 conversion (FP64 pipe) and one
+        // store for the warp's rows
+        float mine = 0.f;
 #pragma unroll
         for (int u = 0; u < RW; ++u) {
             float v = pv[u] * xv[u];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0 && r0 + u < a.n) {
-                z[r0 + u] = (double)v;
-                if (z32) z32[r0 + u] = v;
-            }
+            if (lane == u) mine = v;
+        }
+        if (lane < RW && r0 + lane < a.n) {
+            z[r0 + lane] = (double)mine;
+            if (z32) z32[r0 + lane] = mine;
         }
     }
 }
