@@ -1103,7 +1103,7 @@ int solve_impl(bae_problem* P, int nb, const double* f, const double* g, const b
     int* d_bad = P->ws().arnI.need(4);
     BAE_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int), st));
     kr_nonfinite(d_f, (long long)nb * n3, P->geo.flags, n3, d_bad, st);
-    kr_nonfinite(d_g, (long long)nb * ng, nullptr, 1, d_bad, st);
+    kr_nonfinite(d_g, (long long)nb * ng, nullptr, ng, d_bad, st);
     std::vector<bae_stats> st_local(nb);
     for (auto& s : st_local) {
         std::memset(&s, 0, sizeof(s));

@@ -89,6 +89,7 @@ namespace {
 template <typename T>
 __global__ void k_closure_gather(const T* v, long long v_stride, const int* gm, const int* partner,
                                  const double* t, int n, double* out, long long out_stride, const int* active) {
+    wait_prior_grid();
     const int b = blockIdx.y;
     if (active && !active[b]) return;
     const T* vb = v + b * v_stride;
@@ -107,6 +108,7 @@ __global__ void k_direct_rows(const W* __restrict__ w, long long w_stride, const
                               const int* x_row, long long x_row_stride, const int* __restrict__ gp,
                               const int* __restrict__ pu, const double* __restrict__ t, long long n_gm,
                               long long n_unk, const int* active, Y* y, long long y_stride) {
+    wait_prior_grid();
     const int b = blockIdx.y;
     if (active && !active[b]) return;
     const double* xb = x + b * x_stride + (x_row ? (long long)x_row[b] * x_row_stride : 0);
@@ -128,6 +130,7 @@ __global__ void k_direct_rows(const W* __restrict__ w, long long w_stride, const
 // unknown into the reconstructed grid function
 __global__ void k_scatter_gm(const double* q, long long q_stride, const int* __restrict__ gm, long long n,
                              double* u, long long n3) {
+    wait_prior_grid();
     const int b = blockIdx.y;
     for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < n; r += (long long)gridDim.x * blockDim.x)
         u[b * n3 + gm[r]] = q[b * q_stride + r];
@@ -136,6 +139,7 @@ __global__ void k_scatter_gm(const double* q, long long q_stride, const int* __r
 template <typename T>
 __global__ void k_volume_combine(const T* v, const double* add, const uint8_t* flags, long long n3, double* u,
                                  int v_swap, int N) {
+    wait_prior_grid();
     const int b = blockIdx.y;
     for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < n3; x += (long long)gridDim.x * blockDim.x) {
         const bool np = (flags[x] & 3) != 0;   // M+ or gamma-
@@ -148,6 +152,35 @@ __global__ void k_volume_combine(const T* v, const double* add, const uint8_t* f
     }
 }
 
+// The same for v_swap = 2 (v has axes 0 and 2 swapped): 32 x 32 tiles (i, k) of
+// one j through shared memory, so that v is read and u written contiguously.
+// Only the tiles with nodes of N+ read v. Grid: (k tile, i tile, j + N b).
+template <typename T>
+__global__ void __launch_bounds__(256) k_volume_combine_swapped(const T* v, const double* add, const uint8_t* flags,
+                                                                long long n3, double* u, int N) {
+    wait_prior_grid();
+    __shared__ double tile[32][33];
+    const int b = blockIdx.z / N, j = blockIdx.z % N, i0 = blockIdx.y * 32, k0 = blockIdx.x * 32;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    bool np[4], any = false;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {   // M+ or gamma-
+        np[q] = (flags[((long long)(i0 + ty + 8 * q) * N + j) * N + k0 + tx] & 3) != 0;
+        any |= np[q];
+    }
+    if (__syncthreads_or(any)) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const long long x = b * n3 + ((long long)(k0 + ty + 8 * q) * N + j) * N + i0 + tx;
+            tile[ty + 8 * q][tx] = (add ? add[x] : 0.0) + (double)v[x];
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        u[b * n3 + ((long long)(i0 + ty + 8 * q) * N + j) * N + k0 + tx] = np[q] ? tile[tx][ty + 8 * q] : 0.0;
+}
+
 __global__ void k_to_dsf(const double* in, long long n, dsf* out) {
     for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < n; x += (long long)gridDim.x * blockDim.x)
         out[x] = dsf(in[x]);
@@ -155,6 +188,7 @@ __global__ void k_to_dsf(const double* in, long long n, dsf* out) {
 
 template <typename T>
 __global__ void k_widen(const T* v, long long n, double* out) {
+    wait_prior_grid();
     for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < n; x += (long long)gridDim.x * blockDim.x)
         out[x] = (double)v[x];
 }
@@ -216,7 +250,8 @@ void closure_gather(const T* v, long long v_stride, const int* gm, const int* pa
                     int n, int nbatch, double* out, long long out_stride, cudaStream_t st, const int* active) {
     if (n == 0) return;
     dim3 grid(ceil_div(n, 256) < 1184 ? ceil_div(n, 256) : 1184, nbatch);
-    BAE_LAUNCH(kname<T>("closure_gather.f32", "closure_gather.f64", "closure_gather.f64"), st, k_closure_gather<T><<<grid, 256, 0, st>>>(v, v_stride, gm, partner, t, n, out, out_stride, active));
+    BAE_LAUNCH(kname<T>("closure_gather.f32", "closure_gather.f64", "closure_gather.f64"), st,
+               launch_pdl(k_closure_gather<T>, grid, 256, 0, st, v, v_stride, gm, partner, t, n, out, out_stride, active));
 }
 
 __global__ void k_mask_bit(const uint8_t* __restrict__ flags, long long n, uint8_t bit, uint8_t* __restrict__ out) {
@@ -234,27 +269,32 @@ void direct_rows(const W* w, long long w_stride, const double* x, long long x_st
                  long long x_row_stride, const int* gp, const int* pu, const double* t, long long n_gm, long long n_unk,
                  int nb, const int* active, Y* y, long long y_stride, cudaStream_t st) {
     dim3 grid(ceil_div(n_unk, 256) < 1184 ? ceil_div(n_unk, 256) : 1184, nb);
-    BAE_LAUNCH("k_direct_rows", st, k_direct_rows<W, Y><<<grid, 256, 0, st>>>(w, w_stride, x, x_stride, x_row, x_row_stride,
+    BAE_LAUNCH("k_direct_rows", st, launch_pdl(k_direct_rows<W, Y>, grid, 256, 0, st, w, w_stride, x, x_stride, x_row, x_row_stride,
                                                                               gp, pu, t, n_gm, n_unk, active, y, y_stride));
 }
 
 void scatter_gm(const double* q, long long q_stride, const int* gm, long long n, int nb, double* u, long long n3,
                 cudaStream_t st) {
     dim3 grid(ceil_div(n, 256) < 1184 ? ceil_div(n, 256) : 1184, nb);
-    BAE_LAUNCH("k_scatter_gm", st, k_scatter_gm<<<grid, 256, 0, st>>>(q, q_stride, gm, n, u, n3));
+    BAE_LAUNCH("k_scatter_gm", st, launch_pdl(k_scatter_gm, grid, 256, 0, st, q, q_stride, gm, n, u, n3));
 }
 
 template <typename T>
 void volume_combine(const T* v, const double* add, const uint8_t* flags, long long n3, int nbatch,
                     double* u, cudaStream_t st, int v_swap, int N) {
     BAE_REQUIRE(v_swap == 0 || (long long)N * N * N == n3, BAE_ERR_INVALID_ARG, "volume_combine: N must match n3");
+    if (v_swap == 2 && N % 32 == 0 && (long long)N * nbatch <= 65535) {
+        BAE_LAUNCH("k_volume_combine", st,
+                   launch_pdl(k_volume_combine_swapped<T>, dim3(N / 32, N / 32, N * nbatch), 256, 0, st, v, add, flags, n3, u, N));
+        return;
+    }
     dim3 grid(ceil_div(n3, 256) < 2432 ? ceil_div(n3, 256) : 2432, nbatch);
-    BAE_LAUNCH("k_volume_combine", st, k_volume_combine<T><<<grid, 256, 0, st>>>(v, add, flags, n3, u, v_swap, N));
+    BAE_LAUNCH("k_volume_combine", st, launch_pdl(k_volume_combine<T>, grid, 256, 0, st, v, add, flags, n3, u, v_swap, N));
 }
 
 template <typename T>
 void widen(const T* v, long long n, double* out, cudaStream_t st) {
-    BAE_LAUNCH("k_widen", st, k_widen<T><<<ceil_div(n, 256) < 2432 ? ceil_div(n, 256) : 2432, 256, 0, st>>>(v, n, out));
+    BAE_LAUNCH("k_widen", st, launch_pdl(k_widen<T>, dim3(ceil_div(n, 256) < 2432 ? ceil_div(n, 256) : 2432), 256, 0, st, v, n, out));
 }
 
 void to_dsf(const double* in, long long n, dsf* out, cudaStream_t st) {

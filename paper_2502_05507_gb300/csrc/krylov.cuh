@@ -13,7 +13,8 @@ namespace bae {
 int krylov_chunks(int n);
 
 // *d_flag |= 1 if some x[i] is not finite, counting only i whose
-// flags[i % period] has bit 0 (M+) when flags is not null
+// flags[i % period] has bit 0 (M+) when flags is not null; n a multiple of
+// period, at most 65535 of them
 void kr_nonfinite(const double* x, long long n, const uint8_t* flags, long long period, int* d_flag,
                   cudaStream_t st);
 
