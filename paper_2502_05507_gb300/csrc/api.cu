@@ -1610,11 +1610,6 @@ int bae_problem_create(bae_ctx* ctx, int N, double h, const double origin[3], co
         try {
             P->spec = ctx->spectrum(N, P->s);
             ctx->twiddles(2 * N);   // built here so that later applies allocate nothing
-            P->box = conv_box(P->geo);
-            if (P->box.nt != N) {
-                P->spec_win = ctx->spectrum(P->box.nt, P->s, 2);
-                ctx->twiddles(2 * P->box.nt);
-            }
         // the Schwarz rows of the default (mixed, preconditioned) solve, built
         // on the side stream from here on; a solve waits for them only when it
         // uses them
@@ -1623,6 +1618,14 @@ int bae_problem_create(bae_ctx* ctx, int N, double h, const double origin[3], co
         build_precond(P->geo, P->s, P->spec->near, P->pre, ctx->side);
         BAE_CUDA(cudaEventRecord(ctx->join_ev, ctx->side));
         P->pre.pending = true;
+        // beside them on the main stream (N = 128 torus: 125 us of rows beside
+        // 80 us of view)
+        build_geometry_view(P->geo, ctx->stream);
+        P->box = conv_box(P->geo);
+        if (P->box.nt != N) {
+            P->spec_win = ctx->spectrum(P->box.nt, P->s, 2);
+            ctx->twiddles(2 * P->box.nt);
+        }
         if (P->direct()) {
             const long long nu = P->geo.n_unk;
             std::vector<int> io(nu);

@@ -51,11 +51,11 @@ __device__ int block_exclusive_scan(int v, int* s_warp) {
 }
 
 // ------------------------------------------------------------ point sets
-// One CTA per grid line (i, j), its threads over k.
-constexpr int LINE_T = 128;
+// A warp per grid line (i, j), its lanes over k; N^2 lines are a multiple of
+// the eight warps of a CTA (N a power of two, at least 8).
 
 // slots of the small device record the host reads once
-// (I_NGM .. I_MP: the totals of the scans, in the order of their arrays)
+// (I_NGM .. I_GP: the totals of the scans, in the order of their arrays)
 enum { I_ERR = 0, I_FIRST, I_LAST, I_NGM, I_NSRC, I_NTERM, I_GP, I_MP, I_FIRSTY, I_LASTY, I_FIRSTZ, I_LASTZ,
        I_COUNT };
 
@@ -64,126 +64,194 @@ __device__ __forceinline__ bool in_grid(int i, int j, int k, int N) {
 }
 
 // phi < 0 and phi not finite, by integer operations: a float64 comparison
-// holds GB300's FP64 pipe for 64 cycles per warp, and seven of them per node
-// were what k_nbits took (N = 128: 42 us)
+// holds GB300's FP64 pipe for 64 cycles per warp
 __device__ __forceinline__ bool negative(double p) {
     const int hi = __double2hiint(p);
     return hi < 0 && (((hi & 0x7fffffff) | __double2loint(p)) != 0);
 }
 __device__ __forceinline__ bool not_finite(double p) { return (__double2hiint(p) & 0x7ff00000) == 0x7ff00000; }
 
-// atomicMax, left out where the value is there already (a stale read only
-// costs the atomic): thousands of lines raise the same few maxima
-__device__ __forceinline__ void raise(int* m, int v) {
-    if (*reinterpret_cast<volatile int*>(m) < v) atomicMax(m, v);
+// The node classes are formed as bit words: word w of a line holds the nodes
+// 32 w .. 32 w + 31 (N < 32: one word of N bits). As one CTA per line with six
+// byte loads per node the two passes took 40 + 47 us at N = 128, almost all of
+// it instruction issue; three passes over words take a seventh of that.
+__device__ __forceinline__ int words(int N) { return (N + 31) >> 5; }
+
+// the word of the same k's in a neighbouring line (di, dj), 0 outside the box
+__device__ __forceinline__ unsigned line_word(const unsigned* __restrict__ m, int i, int j, int w, int N) {
+    return (unsigned)i < (unsigned)N && (unsigned)j < (unsigned)N ? m[(i * N + j) * words(N) + w] : 0u;
 }
 
-// bits per node from phi: bit0 in M+ (phi < 0), bit1 an M+ neighbour, bit2
-// a neighbour outside M+ (nodes outside the box count as exterior); a phi that
-// is not finite ends the problem, whatever its bits
-__global__ void __launch_bounds__(LINE_T) k_nbits(const double* __restrict__ phi, int N, uint8_t* __restrict__ nb,
-                                                 int* __restrict__ info) {
-    const int line = blockIdx.x, i = line / N, j = line - i * N;
-    const long long base = (long long)line * N;
-    for (int k = threadIdx.x; k < N; k += blockDim.x) {
-        const double p = phi[base + k];
-        if (not_finite(p)) atomicOr(info + I_ERR, 1);
-        bool h = false, e = false;
-        for (int d = 0; d < 6; ++d) {
-            const int ii = i + c_dir[d][0], jj = j + c_dir[d][1], kk = k + c_dir[d][2];
-            if (in_grid(ii, jj, kk, N) && negative(phi[((long long)ii * N + jj) * N + kk])) h = true;
-            else e = true;
-        }
-        nb[base + k] = (uint8_t)((negative(p) ? 1 : 0) | (h ? 2 : 0) | (e ? 4 : 0));
-    }
+// bit k of q[d] = bit of the neighbour of node k in direction d (order of
+// c_dir; 0 outside the box): the four neighbouring lines' words, and the
+// word itself moved by one node with the adjoining words' end bits
+__device__ __forceinline__ void neighbour_words(const unsigned* __restrict__ m, int i, int j, int w, int N,
+                                                unsigned q[6]) {
+    const unsigned* row = m + (i * N + j) * words(N);
+    const unsigned me = row[w];
+    q[0] = line_word(m, i + 1, j, w, N);
+    q[1] = line_word(m, i - 1, j, w, N);
+    q[2] = line_word(m, i, j + 1, w, N);
+    q[3] = line_word(m, i, j - 1, w, N);
+    q[4] = (me >> 1) | (w + 1 < words(N) ? row[w + 1] << 31 : 0u);
+    q[5] = (me << 1) | (w > 0 ? row[w - 1] >> 31 : 0u);
 }
 
-// Node flags from the bits of the node and its six neighbours: M+ (bit0),
-// gamma- = outside M+ with an M+ neighbour (bit1), gamma+ = M+ with an
-// exterior neighbour (bit2), D-node = outside N+ = M+ and gamma-, next to a
-// gamma- node (bit3), and for gamma- nodes |D_n| = the neighbours outside
-// N+ (bits 4-6). Per line: the gamma- nodes, the sources (flags & src_mask)
-// and their stencil terms (a D-node: one per gamma- neighbour; a gamma- node:
-// 1, or with `direct` 1 + its neighbours in gamma = gamma- u gamma+), the
-// gamma+ nodes, the M+ nodes; the range of source planes goes to info.
-__global__ void __launch_bounds__(LINE_T) k_flags_lines(const uint8_t* __restrict__ nb, int N, int src_mask,
-                                                       bool direct, uint8_t* __restrict__ flags,
-                                                       int* __restrict__ cnt_gm, int* __restrict__ cnt_src,
-                                                       int* __restrict__ cnt_term, int* __restrict__ cnt_gp,
-                                                       int* __restrict__ cnt_mp, int* __restrict__ info) {
-    __shared__ int s_red[5][LINE_T / 32];
-    const int line = blockIdx.x, i = line / N, j = line - i * N;
-    const long long base = (long long)line * N;
-    int c[5] = {0, 0, 0, 0, 0};   // gamma-, sources, terms, gamma+, M+
-    int klo = N, khi = -1;        // k range of this thread's sources
-    for (int k = threadIdx.x; k < N; k += blockDim.x) {
-        const int me = nb[base + k];
-        bool out_nb = false;
-        int n_out = 0, n_gm = 0, n_gam = 0;
-        for (int d = 0; d < 6; ++d) {
-            const int ii = i + c_dir[d][0], jj = j + c_dir[d][1], kk = k + c_dir[d][2];
-            const int q = in_grid(ii, jj, kk, N) ? nb[((long long)ii * N + jj) * N + kk] : 0;
-            if (!(q & 1)) out_nb = true;
-            if (!(q & 3)) ++n_out;               // not in N+
-            if (!(q & 1) && (q & 2)) ++n_gm;     // a gamma- node
-            if ((q & 1) ? (q & 4) : (q & 2)) ++n_gam;   // gamma+ or gamma-
-        }
-        const bool in = me & 1, gm = !in && (me & 2);
-        const bool gp = in && out_nb;
-        const bool dnode = !in && !gm && n_gm > 0;
-        const bool face = (i == 0 || j == 0 || k == 0 || i == N - 1 || j == N - 1 || k == N - 1);
-        if ((gm || in) && face) atomicOr(info + I_ERR, 2);
-        const int f = (in ? 1 : 0) | (gm ? 2 : 0) | (gp ? 4 : 0) | (dnode ? 8 : 0) | ((gm ? n_out : 0) << 4);
-        flags[base + k] = (uint8_t)f;
-        const bool src = (f & src_mask) != 0;
-        if (src) {
-            klo = min(klo, k);
-            khi = max(khi, k);
-        }
-        c[0] += gm;
-        c[1] += src;
-        c[2] += src ? (gm ? (direct ? 1 + n_gam : 1) : n_gm) : 0;
-        c[3] += gp;
-        c[4] += in;
-    }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+// M+ (phi < 0) as words; a phi that is not finite ends the problem, whatever its
+// bit. A warp takes four words, their loads in flight together.
+__global__ void __launch_bounds__(256) k_inside(const double* __restrict__ phi, int N, unsigned* __restrict__ in,
+                                               int* __restrict__ info) {
+    constexpr int U = 4;
+    const int nw = words(N), lane = threadIdx.x & 31, total = N * N * nw;
+    const int w0 = U * (blockIdx.x * 8 + (threadIdx.x >> 5));
+    double p[U];
 #pragma unroll
-    for (int e = 0; e < 5; ++e) {
-        const int v = __reduce_add_sync(0xffffffffu, c[e]);
-        if (lane == 0) s_red[e][w] = v;
+    for (int u = 0; u < U; ++u) {
+        const int word = w0 + u, line = word / nw, k = 32 * (word - line * nw) + lane;
+        p[u] = word < total && k < N ? phi[(long long)line * N + k] : 1.0;
     }
-    klo = __reduce_min_sync(0xffffffffu, klo);
-    khi = __reduce_max_sync(0xffffffffu, khi);
-    if (lane == 0 && khi >= 0) {
-        raise(info + I_FIRSTZ, N - klo);
-        raise(info + I_LASTZ, khi + 1);
+    unsigned mine = 0;
+    bool bad = false;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        bad |= not_finite(p[u]);
+        const unsigned b = __ballot_sync(0xffffffffu, negative(p[u]));
+        if (lane == u) mine = b;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int t[5] = {0, 0, 0, 0, 0};
-        for (int e = 0; e < 5; ++e)
-            for (int x = 0; x < (int)(blockDim.x >> 5); ++x) t[e] += s_red[e][x];
-        cnt_gm[line] = t[0];
-        cnt_src[line] = t[1];
-        cnt_term[line] = t[2];
-        cnt_gp[line] = t[3];
-        cnt_mp[line] = t[4];
-        if (t[1]) {
-            raise(info + I_FIRST, N - i);
-            raise(info + I_LAST, i + 1);
-            raise(info + I_FIRSTY, N - j);
-            raise(info + I_LASTY, j + 1);
+    if (bad) atomicOr(info + I_ERR, 1);
+    if (lane < U && w0 + lane < total) in[w0 + lane] = mine;
+}
+
+// gamma- = outside M+ with an M+ neighbour, and gamma+ = M+ with an exterior
+// neighbour (nodes outside the box count as exterior); a thread per word
+__global__ void __launch_bounds__(256) k_gamma_words(const unsigned* __restrict__ in, int N, unsigned* __restrict__ gm,
+                                                    unsigned* __restrict__ gp) {
+    const int nw = words(N), word = blockIdx.x * 256 + threadIdx.x;
+    if (word >= N * N * nw) return;
+    const int line = word / nw, w = word - line * nw, i = line / N, j = line - i * N;
+    const unsigned valid = N < 32 ? (1u << N) - 1u : 0xffffffffu, me = in[word];
+    unsigned q[6];
+    neighbour_words(in, i, j, w, N, q);
+    gm[word] = valid & ~me & (q[0] | q[1] | q[2] | q[3] | q[4] | q[5]);
+    gp[word] = me & ~(q[0] & q[1] & q[2] & q[3] & q[4] & q[5]);
+}
+
+// per line: M+ nodes (at most 256), N - the first and 1 + the last k of its
+// sources (0, 0: none), nine bits each
+__device__ __forceinline__ int line_box(int mp, int first, int last) { return mp | (first << 9) | (last << 18); }
+
+// Node flags: M+ (bit0), gamma- (bit1), gamma+ (bit2), D-node = outside N+ =
+// M+ and gamma-, next to a gamma- node (bit3), and for gamma- nodes |D_n| =
+// the neighbours outside N+ (bits 4-6). A warp per line; lane = node of the
+// word. Per line, by population counts that every lane forms: the gamma-
+// nodes, the sources (flags & src_mask) and their stencil terms (a D-node: one
+// per gamma- neighbour; a gamma- node: 1, or with `direct` 1 + its neighbours
+// in gamma = gamma- u gamma+), the gamma+ nodes, and in one int the M+ nodes
+// and the k range of the sources (line_box); k_scan_lines forms totals and
+// ranges from them.
+__global__ void __launch_bounds__(256) k_flags_lines(const unsigned* __restrict__ in, const unsigned* __restrict__ gmw,
+                                                    const unsigned* __restrict__ gpw, int N, int src_mask,
+                                                    bool direct, uint8_t* __restrict__ flags,
+                                                    int* __restrict__ cnt_gm, int* __restrict__ cnt_src,
+                                                    int* __restrict__ cnt_term, int* __restrict__ cnt_gp,
+                                                    int* __restrict__ cnt_box, int* __restrict__ info) {
+    const int nw = words(N), lane = threadIdx.x & 31;
+    const int line = blockIdx.x * 8 + (threadIdx.x >> 5), i = line / N, j = line - i * N;
+    int c_gm = 0, c_src = 0, c_term = 0, c_gp = 0, c_in = 0, klo = N, khi = -1;
+    unsigned touch = 0;   // gamma- and M+ nodes on a face of the box
+    for (int w = 0; w < nw; ++w) {
+        const unsigned I = in[line * nw + w], G = gmw[line * nw + w], P = gpw[line * nw + w];
+        unsigned g[6], a[6];
+        neighbour_words(gmw, i, j, w, N, g);
+        if (!(I | G | g[0] | g[1] | g[2] | g[3] | g[4] | g[5])) {   // the most words: no M+, gamma- or D-node
+            if (32 * w + lane < N) flags[(long long)line * N + 32 * w + lane] = 0;
+            continue;
         }
+        neighbour_words(in, i, j, w, N, a);
+        const unsigned D = ~I & ~G & (g[0] | g[1] | g[2] | g[3] | g[4] | g[5]) & (N < 32 ? (1u << N) - 1u : 0xffffffffu);
+        const unsigned S = (src_mask & 2 ? G : 0u) | (src_mask & 8 ? D : 0u);
+        int n_out = 6;
+#pragma unroll
+        for (int d = 0; d < 6; ++d) {
+            c_term += __popc(S & D & g[d]);
+            n_out -= ((a[d] | g[d]) >> lane) & 1;
+        }
+        if (direct && G) {
+            unsigned p[6];
+            neighbour_words(gpw, i, j, w, N, p);
+#pragma unroll
+            for (int d = 0; d < 6; ++d) c_term += __popc(G & (g[d] | p[d]));
+        }
+        c_term += __popc(S & G);
+        c_gm += __popc(G);
+        c_src += __popc(S);
+        c_gp += __popc(P);
+        c_in += __popc(I);
+        if (S) {
+            klo = min(klo, 32 * w + __ffs(S) - 1);
+            khi = 32 * w + 31 - __clz(S);
+        }
+        if (i == 0 || j == 0 || i == N - 1 || j == N - 1) touch |= I | G;
+        if (w == 0) touch |= (I | G) & 1u;
+        if (w == nw - 1) touch |= (I | G) & (1u << ((N - 1) & 31));
+        const int f = ((I >> lane) & 1) | (((G >> lane) & 1) << 1) | (((P >> lane) & 1) << 2) | (((D >> lane) & 1) << 3) |
+                      ((G >> lane) & 1 ? n_out << 4 : 0);
+        if (32 * w + lane < N) flags[(long long)line * N + 32 * w + lane] = (uint8_t)f;
+    }
+    if (lane == 0) {
+        if (touch) atomicOr(info + I_ERR, 2);
+        cnt_gm[line] = c_gm;
+        cnt_src[line] = c_src;
+        cnt_term[line] = c_term;
+        cnt_gp[line] = c_gp;
+        cnt_box[line] = line_box(c_in, N - klo, khi + 1);
     }
 }
 
 // In-place exclusive scans of the per-line counts (nl + 1 entries, the last
-// one becomes the total; nl a multiple of SCAN_E), one CTA each; totals to
-// info.
-__global__ void __launch_bounds__(1024) k_scan_lines(int* c0, int* c1, int* c2, int* c3, int* c4, int nl, int* info) {
+// one becomes the total; nl = N^2 a multiple of SCAN_E), one CTA each; totals to
+// info, and from the source counts (c1) the range of their i and j. CTA 4: the
+// M+ total and the k range of the sources from the lines' boxes (not scanned).
+__device__ __forceinline__ int block_max(int v, int* s_warp) {
+    v = __reduce_max_sync(0xffffffffu, v);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = v;
+    __syncthreads();
+    return __reduce_max_sync(0xffffffffu, s_warp[threadIdx.x & 31]);   // 32 warps
+}
+__global__ void __launch_bounds__(1024) k_scan_lines(int* c0, int* c1, int* c2, int* c3, const int* box, int N,
+                                                     int* info) {
+    const int nl = N * N, lg = 31 - __clz(N);
     __shared__ int s_warp[33];
     __shared__ int s_carry;
-    int* arr = blockIdx.x == 0 ? c0 : (blockIdx.x == 1 ? c1 : (blockIdx.x == 2 ? c2 : (blockIdx.x == 3 ? c3 : c4)));
+    if (blockIdx.x == 4) {
+        int mp = 0, first = 0, last = 0;
+        auto take = [&](int v) {
+            mp += v & 511;
+            first = max(first, (v >> 9) & 511);
+            last = max(last, v >> 18);
+        };
+#pragma unroll 4
+        for (int l = threadIdx.x; l < nl / 4; l += blockDim.x) {
+            const int4 q = reinterpret_cast<const int4*>(box)[l];
+            take(q.x);
+            take(q.y);
+            take(q.z);
+            take(q.w);
+        }
+        block_exclusive_scan(mp, s_warp);
+        const int total = s_warp[32];
+        first = block_max(first, s_warp);
+        last = block_max(last, s_warp);
+        if (threadIdx.x == 0) {
+            info[I_MP] = total;
+            info[I_FIRSTZ] = first;
+            info[I_LASTZ] = last;
+        }
+        return;
+    }
+    int* arr = blockIdx.x == 0 ? c0 : (blockIdx.x == 1 ? c1 : (blockIdx.x == 2 ? c2 : c3));
+    int r[4] = {0, 0, 0, 0};   // N - first and 1 + last i, then j, of the lines with a count
     if (threadIdx.x == 0) s_carry = 0;
     __syncthreads();
     for (int base = 0; base < nl; base += blockDim.x * SCAN_E) {
@@ -198,6 +266,20 @@ __global__ void __launch_bounds__(1024) k_scan_lines(int* c0, int* c1, int* c2, 
             v[e + 2] = q.z;
             v[e + 3] = q.w;
             tot += q.x + q.y + q.z + q.w;
+        }
+        // eight entries lie on one line of i (N a power of two, at least 8)
+#pragma unroll
+        for (int e = 0; e < SCAN_E; e += 8) {
+            unsigned m = 0;
+#pragma unroll
+            for (int x = 0; x < 8; ++x) m |= v[e + x] ? 1u << x : 0u;
+            if (m) {
+                const int i = (b0 + e) >> lg, j = (b0 + e) & (N - 1);
+                r[0] = max(r[0], N - i);
+                r[1] = max(r[1], i + 1);
+                r[2] = max(r[2], N - (j + __ffs(m) - 1));
+                r[3] = max(r[3], j + 32 - __clz(m));
+            }
         }
         const int ex = block_exclusive_scan(tot, s_warp);
         int run = ex + s_carry;
@@ -215,67 +297,86 @@ __global__ void __launch_bounds__(1024) k_scan_lines(int* c0, int* c1, int* c2, 
         arr[nl] = s_carry;
         info[I_NGM + blockIdx.x] = s_carry;
     }
+    if (blockIdx.x == 1) {
+        const int slot[4] = {I_FIRST, I_LAST, I_FIRSTY, I_LASTY};
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const int v = block_max(r[x], s_warp);
+            if (threadIdx.x == 0) info[slot[x]] = v;
+        }
+    }
 }
 
-// The lists in lexicographic order: per line, the CTA scans its nodes
-// (gamma-, source and term counts packed in one int: at most 256, 256 and
-// 1792 per line; gamma+ in a second scan) from the line's offsets.
+// inclusive sum over the lanes of a warp
+__device__ __forceinline__ int warp_inclusive_scan(int x) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    return x;
+}
+
+// The lists in lexicographic order: a warp per line, which ranks its nodes by
+// ballots (and the terms by a shuffle scan) from the line's offsets; a line
+// without sources and gamma+ nodes ends at once.
 // node_of[x] = index of gamma- node x, n_gm + index of gamma+ node x (set
 // only there: the unknown numbers of the direct formulation); term_off[s] =
 // first term of source s.
-__global__ void __launch_bounds__(LINE_T) k_scatter_lines(const uint8_t* __restrict__ flags, int N, int src_mask,
-                                                         bool direct, const int* __restrict__ off_gm,
-                                                         const int* __restrict__ off_src,
-                                                         const int* __restrict__ off_term,
-                                                         const int* __restrict__ off_gp, const int* __restrict__ info,
-                                                         int* __restrict__ gm, int* __restrict__ gp,
-                                                         int* __restrict__ node_of, int* __restrict__ src_lin,
-                                                         int* __restrict__ term_off) {
-    __shared__ int s_warp[33];
-    const int line = blockIdx.x, i = line / N, j = line - i * N;
-    if (line == (int)gridDim.x - 1 && threadIdx.x == 0) term_off[info[I_NSRC]] = info[I_NTERM];
+__global__ void __launch_bounds__(256) k_scatter_lines(const uint8_t* __restrict__ flags, int N, int src_mask,
+                                                      bool direct, const int* __restrict__ off_gm,
+                                                      const int* __restrict__ off_src,
+                                                      const int* __restrict__ off_term,
+                                                      const int* __restrict__ off_gp, const int* __restrict__ info,
+                                                      int* __restrict__ gm, int* __restrict__ gp,
+                                                      int* __restrict__ node_of, int* __restrict__ src_lin,
+                                                      int* __restrict__ term_off) {
+    const int lane = threadIdx.x & 31;
+    const int line = blockIdx.x * 8 + (threadIdx.x >> 5), i = line / N, j = line - i * N;
+    if (line == N * N - 1 && lane == 0) term_off[info[I_NSRC]] = info[I_NTERM];
     int pg = off_gm[line], ps = off_src[line], pt = off_term[line], pp = off_gp[line];
     const int ngm = info[I_NGM];
-    if (ps == off_src[line + 1] && pp == off_gp[line + 1]) return;   // nothing on this line: the whole CTA
+    if (ps == off_src[line + 1] && pp == off_gp[line + 1]) return;   // nothing on this line: the whole warp
     const int base = line * N;
-    for (int k0 = 0; k0 < N; k0 += blockDim.x) {
-        const int k = k0 + (int)threadIdx.x;
-        int g = 0, s = 0, nt = 0, p = 0;
-        if (k < N) {
-            const int f = flags[base + k];
-            g = (f >> 1) & 1;
-            p = (f >> 2) & 1;
-            s = (f & src_mask) != 0;
-            if (s) {
-                const int want = g ? 6 : 2;   // gamma- and gamma+ neighbours, or gamma- neighbours
-                nt = g ? 1 : 0;
-                if (!g || direct)
-                    for (int d = 0; d < 6; ++d) {
-                        const int ii = i + c_dir[d][0], jj = j + c_dir[d][1], kk = k + c_dir[d][2];
-                        if (in_grid(ii, jj, kk, N) && (flags[(ii * N + jj) * N + kk] & want)) ++nt;
-                    }
-            }
+    const unsigned below = (1u << lane) - 1u;
+    for (int k0 = 0; k0 < N; k0 += 32) {
+        const int k = k0 + lane;
+        const int f = k < N ? flags[base + k] : 0;
+        const bool g = f & 2, p = f & 4, s = (f & src_mask) != 0;
+        const unsigned mg = __ballot_sync(0xffffffffu, g), mp = __ballot_sync(0xffffffffu, p);
+        const unsigned ms = __ballot_sync(0xffffffffu, s);
+        if (!(ms | mp)) continue;
+        int nt = 0;
+        if (s) {
+            const int want = g ? 6 : 2;   // gamma- and gamma+ neighbours, or gamma- neighbours
+            nt = g ? 1 : 0;
+            if (!g || direct)
+                for (int d = 0; d < 6; ++d) {
+                    const int ii = i + c_dir[d][0], jj = j + c_dir[d][1], kk = k + c_dir[d][2];
+                    if (in_grid(ii, jj, kk, N) && (flags[(ii * N + jj) * N + kk] & want)) ++nt;
+                }
         }
-        const int ex = block_exclusive_scan(g | (s << 10) | (nt << 20), s_warp);
-        const int tot = s_warp[32];
-        const int exp_ = block_exclusive_scan(p, s_warp);
-        const int totp = s_warp[32];
+        const int et = warp_inclusive_scan(nt);
         if (p) {
-            gp[pp + exp_] = base + k;
-            node_of[base + k] = ngm + pp + exp_;
+            const int x = pp + __popc(mp & below);
+            gp[x] = base + k;
+            node_of[base + k] = ngm + x;
         }
-        pp += totp;
         if (g) {
-            gm[pg + (ex & 1023)] = base + k;
-            node_of[base + k] = pg + (ex & 1023);
+            const int x = pg + __popc(mg & below);
+            gm[x] = base + k;
+            node_of[base + k] = x;
         }
         if (s) {
-            src_lin[ps + ((ex >> 10) & 1023)] = base + k;
-            term_off[ps + ((ex >> 10) & 1023)] = pt + (ex >> 20);
+            const int x = ps + __popc(ms & below);
+            src_lin[x] = base + k;
+            term_off[x] = pt + et - nt;
         }
-        pg += tot & 1023;
-        ps += (tot >> 10) & 1023;
-        pt += tot >> 20;
+        pp += __popc(mp);
+        pg += __popc(mg);
+        ps += __popc(ms);
+        pt += __shfl_sync(0xffffffffu, et, 31);
     }
 }
 
@@ -421,74 +522,60 @@ __global__ void k_src_map(const int* __restrict__ src_lin, int ns, int* __restri
 }
 
 // Per line of the swapped grid: the number of its sources (swapped flags &
-// src_mask: the nodes the plain recipe lists) and of their terms.
-__global__ void __launch_bounds__(LINE_T) k_view_count(const uint8_t* __restrict__ vflags, int N, int sw,
-                                                      int src_mask, const int* __restrict__ smap,
-                                                      const int* __restrict__ term_off, int* __restrict__ cnt_src,
-                                                      int* __restrict__ cnt_term) {
-    __shared__ int s_red[2][LINE_T / 32];
-    const long long base = (long long)blockIdx.x * N;
+// src_mask: the nodes the plain recipe lists) and of their terms. A warp per
+// line.
+__global__ void __launch_bounds__(256) k_view_count(const uint8_t* __restrict__ vflags, int N, int sw, int src_mask,
+                                                   const int* __restrict__ smap, const int* __restrict__ term_off,
+                                                   int* __restrict__ cnt_src, int* __restrict__ cnt_term) {
+    const int line = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const long long base = (long long)line * N;
     int c0 = 0, c1 = 0;
-    for (int k = threadIdx.x; k < N; k += blockDim.x) {
+    for (int k = threadIdx.x & 31; k < N; k += 32) {
         const int s = (vflags[base + k] & src_mask) ? smap[swap_axes(base + k, sw, N)] : -1;
         if (s >= 0) {   // every source node of the swapped flags is in the plain recipe
             c0 += 1;
             c1 += term_off[s + 1] - term_off[s];
         }
     }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     c0 = __reduce_add_sync(0xffffffffu, c0);
     c1 = __reduce_add_sync(0xffffffffu, c1);
-    if (lane == 0) {
-        s_red[0][w] = c0;
-        s_red[1][w] = c1;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int t0 = 0, t1 = 0;
-        for (int x = 0; x < (int)(blockDim.x >> 5); ++x) {
-            t0 += s_red[0][x];
-            t1 += s_red[1][x];
-        }
-        cnt_src[blockIdx.x] = t0;
-        cnt_term[blockIdx.x] = t1;
+    if ((threadIdx.x & 31) == 0) {
+        cnt_src[line] = c0;
+        cnt_term[line] = c1;
     }
 }
 
-// The swapped recipe in lexicographic order of the swapped grid: per line,
-// the CTA scans its sources (count in bits 0-10, terms from bit 11) from
-// the line's offsets; vorig[pos] = the source's number in the plain recipe.
-__global__ void __launch_bounds__(LINE_T) k_view_scatter(const uint8_t* __restrict__ vflags, int N, int sw,
-                                                        int src_mask, const int* __restrict__ smap,
-                                                        const int* __restrict__ term_off,
-                                                        const int* __restrict__ off_src,
-                                                        const int* __restrict__ off_term, int n_src, int n_terms,
-                                                        int* __restrict__ vsrc_lin, int* __restrict__ vterm_off,
-                                                        int* __restrict__ vorig) {
-    __shared__ int s_warp[33];
-    const int line = blockIdx.x;
-    if (line == (int)gridDim.x - 1 && threadIdx.x == 0) vterm_off[n_src] = n_terms;
+// The swapped recipe in lexicographic order of the swapped grid: a warp per
+// line ranks its sources from the line's offsets; vorig[pos] = the source's
+// number in the plain recipe.
+__global__ void __launch_bounds__(256) k_view_scatter(const uint8_t* __restrict__ vflags, int N, int sw, int src_mask,
+                                                     const int* __restrict__ smap, const int* __restrict__ term_off,
+                                                     const int* __restrict__ off_src,
+                                                     const int* __restrict__ off_term, int n_src, int n_terms,
+                                                     int* __restrict__ vsrc_lin, int* __restrict__ vterm_off,
+                                                     int* __restrict__ vorig) {
+    const int lane = threadIdx.x & 31;
+    const int line = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (line == N * N - 1 && lane == 0) vterm_off[n_src] = n_terms;
     int ps = off_src[line], pt = off_term[line];
-    if (ps == off_src[line + 1]) return;   // no source on this line: the whole CTA
+    if (ps == off_src[line + 1]) return;   // no source on this line: the whole warp
     const long long base = (long long)line * N;
-    for (int k0 = 0; k0 < N; k0 += blockDim.x) {
-        const int k = k0 + (int)threadIdx.x;
-        int sf = 0, nt = 0, s = -1;
+    for (int k0 = 0; k0 < N; k0 += 32) {
+        const int k = k0 + lane;
+        int nt = 0, s = -1;
         if (k < N && (vflags[base + k] & src_mask)) s = smap[swap_axes(base + k, sw, N)];
-        if (s >= 0) {   // the same nodes as k_view_count counts
-            sf = 1;
-            nt = term_off[s + 1] - term_off[s];
-        }
-        const int ex = block_exclusive_scan(sf | (nt << 11), s_warp);
-        const int tot = s_warp[32];
-        if (sf) {
-            const int pos = ps + (ex & 2047);
+        const unsigned ms = __ballot_sync(0xffffffffu, s >= 0);   // the same nodes as k_view_count counts
+        if (!ms) continue;
+        if (s >= 0) nt = term_off[s + 1] - term_off[s];
+        const int et = warp_inclusive_scan(nt);
+        if (s >= 0) {
+            const int pos = ps + __popc(ms & ((1u << lane) - 1u));
             vsrc_lin[pos] = (int)(base + k);
-            vterm_off[pos] = pt + (ex >> 11);
+            vterm_off[pos] = pt + et - nt;
             vorig[pos] = s;
         }
-        ps += tot & 2047;
-        pt += tot >> 11;
+        ps += __popc(ms);
+        pt += __shfl_sync(0xffffffffu, et, 31);
     }
 }
 
@@ -537,16 +624,16 @@ void build_view(Geometry& g, int sw, int src_mask, Scratch& sc, cudaStream_t st)
     int* off_term = sc.get<int>(nl + 1);
     int* info = sc.get<int>(I_COUNT);
     BAE_LAUNCH("k_view_count", st,
-               k_view_count<<<(unsigned)nl, LINE_T, 0, st>>>(g.cv_flags, N, sw, src_mask, smap, g.term_off, off_src,
+               k_view_count<<<(unsigned)(nl / 8), 256, 0, st>>>(g.cv_flags, N, sw, src_mask, smap, g.term_off, off_src,
                                                              off_term));
-    // blocks 0 and 1 scan the two counts (the other arrays are not read)
-    BAE_LAUNCH("k_scan_lines", st, k_scan_lines<<<2, 1024, 0, st>>>(off_src, off_term, off_src, off_term, off_src, (int)nl, info));
+    // CTAs 0 and 1 scan the two counts (the other arrays are not read)
+    BAE_LAUNCH("k_scan_lines", st, k_scan_lines<<<2, 1024, 0, st>>>(off_src, off_term, off_src, off_term, nullptr, N, info));
     g.cv_src_lin = dev_alloc_n<int>(g.n_src, st);
     g.cv_term_off = dev_alloc_n<int>(g.n_src + 1, st);
     int* vorig = sc.get<int>(std::max(1LL, g.n_src));
     BAE_CUDA(cudaMemsetAsync(vorig, 0xff, std::max(1LL, g.n_src) * sizeof(int), st));
     BAE_LAUNCH("k_view_scatter", st,
-               k_view_scatter<<<(unsigned)nl, LINE_T, 0, st>>>(g.cv_flags, N, sw, src_mask, smap, g.term_off, off_src,
+               k_view_scatter<<<(unsigned)(nl / 8), 256, 0, st>>>(g.cv_flags, N, sw, src_mask, smap, g.term_off, off_src,
                                                                off_term, (int)g.n_src, (int)g.n_terms, g.cv_src_lin,
                                                                g.cv_term_off, vorig));
     g.cv_term_idx = dev_alloc_n<int>(g.n_terms, st);
@@ -591,8 +678,12 @@ void build_geometry(const double* phi, int N, double h, const double origin[3], 
     const long long nl = (long long)N * N;
     int* info = sc.get<int>(I_COUNT);
     BAE_CUDA(cudaMemsetAsync(info, 0, I_COUNT * sizeof(int), st));
-    uint8_t* nbits = sc.get<uint8_t>(n3);
-    BAE_LAUNCH("k_nbits", st, k_nbits<<<(unsigned)nl, LINE_T, 0, st>>>(phi, N, nbits, info));
+    const int n_words = (int)nl * ceil_div(N, 32);
+    unsigned* w_in = sc.get<unsigned>(n_words);
+    unsigned* w_gm = sc.get<unsigned>(n_words);
+    unsigned* w_gp = sc.get<unsigned>(n_words);
+    BAE_LAUNCH("k_inside", st, k_inside<<<ceil_div(n_words, 32), 256, 0, st>>>(phi, N, w_in, info));
+    BAE_LAUNCH("k_gamma_words", st, k_gamma_words<<<ceil_div(n_words, 256), 256, 0, st>>>(w_in, N, w_gm, w_gp));
     const bool direct = layer == BAE_LAYER_DIRECT;
     // gamma- and D-nodes (double layer, direct formulation), or gamma- only
     const int src_mask = layer == BAE_LAYER_SINGLE ? 2 : (2 | 8);
@@ -601,11 +692,11 @@ void build_geometry(const double* phi, int N, double h, const double origin[3], 
     int* off_gm = sc.get<int>(nl + 1);
     int* off_term = sc.get<int>(nl + 1);
     int* off_gp = sc.get<int>(nl + 1);
-    int* off_mp = sc.get<int>(nl + 1);
+    int* box = sc.get<int>(nl);
     BAE_LAUNCH("k_flags_lines", st,
-               k_flags_lines<<<(unsigned)nl, LINE_T, 0, st>>>(nbits, N, src_mask, direct, g.flags, off_gm, g.line_off,
-                                                              off_term, off_gp, off_mp, info));
-    BAE_LAUNCH("k_scan_lines", st, k_scan_lines<<<5, 1024, 0, st>>>(off_gm, g.line_off, off_term, off_gp, off_mp, (int)nl, info));
+               k_flags_lines<<<(unsigned)(nl / 8), 256, 0, st>>>(w_in, w_gm, w_gp, N, src_mask, direct, g.flags, off_gm,
+                                                                 g.line_off, off_term, off_gp, box, info));
+    BAE_LAUNCH("k_scan_lines", st, k_scan_lines<<<5, 1024, 0, st>>>(off_gm, g.line_off, off_term, off_gp, box, N, info));
     int rec[I_COUNT];
     BAE_CUDA(cudaMemcpyAsync(rec, info, sizeof(rec), cudaMemcpyDeviceToHost, st));
     BAE_CUDA(cudaStreamSynchronize(st));
@@ -625,7 +716,7 @@ void build_geometry(const double* phi, int N, double h, const double origin[3], 
     g.src_lin = dev_alloc_n<int>(g.n_src, st);
     g.term_off = dev_alloc_n<int>(g.n_src + 1, st);
     BAE_LAUNCH("k_scatter_lines", st,
-               k_scatter_lines<<<(unsigned)nl, LINE_T, 0, st>>>(g.flags, N, src_mask, direct, off_gm, g.line_off,
+               k_scatter_lines<<<(unsigned)(nl / 8), 256, 0, st>>>(g.flags, N, src_mask, direct, off_gm, g.line_off,
                                                                 off_term, off_gp, info, g.gm, g.gp, g.node_of,
                                                                 g.src_lin, g.term_off));
     // closure
@@ -667,7 +758,13 @@ void build_geometry(const double* phi, int N, double h, const double origin[3], 
     if (!direct && !keep_x)
         for (int ax = 1; ax < 3; ++ax)
             if (10 * (g.ext_hi[ax] - g.ext_lo[ax]) < 9 * (g.ext_hi[sw] - g.ext_lo[sw])) sw = ax;
-    if (sw) build_view(g, sw, src_mask, sc, st);
+    g.view_axis = sw;
+}
+
+void build_geometry_view(Geometry& g, cudaStream_t st) {
+    if (g.view_axis == 0) return;
+    Scratch sc(st);
+    build_view(g, g.view_axis, g.layer == BAE_LAYER_SINGLE ? 2 : (2 | 8), sc, st);
 }
 
 }  // namespace bae

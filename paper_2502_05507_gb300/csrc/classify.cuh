@@ -45,6 +45,7 @@ struct Geometry {
     // when BAE_CONV_AXIS=x). cv_lo/cv_hi is the plane range along that axis;
     // the recipe, the flags and the gathered indices below are the
     // geometry's in the swapped layout (null when cv_swap == 0).
+    int view_axis = 0;   // the axis, cv_swap once build_geometry_view has built the view
     int cv_swap = 0;
     int cv_lo = 0, cv_hi = 0;
     uint8_t* cv_flags = nullptr;
@@ -90,5 +91,10 @@ struct Geometry {
 // s = kappa^2 h^2 (the direct formulation's source stencil uses 6 + s).
 void build_geometry(const double* phi, int N, double h, const double origin[3], int layer, double s,
                     Geometry& g, cudaStream_t st);
+
+// Builds the swapped view of a built geometry (nothing where view_axis is 0).
+// Apart from build_geometry because only the convolutions read it: the Schwarz
+// rows can be started on another stream before it.
+void build_geometry_view(Geometry& g, cudaStream_t st);
 
 }  // namespace bae
