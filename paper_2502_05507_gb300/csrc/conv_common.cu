@@ -146,7 +146,7 @@ __global__ void k_volume_combine(const T* v, const double* add, const uint8_t* f
         double r = 0.0;
         if (np) {
             const long long xv = swap_axes(x, v_swap, N);
-            r = (add ? add[b * n3 + xv] : 0.0) + (double)v[b * n3 + xv];
+            r = (add ? add[b * n3 + xv] : 0.0) + widen(v[b * n3 + xv]);
         }
         u[b * n3 + x] = r;
     }
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(256) k_volume_combine_swapped(const T* v, cons
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const long long x = b * n3 + ((long long)(k0 + ty + 8 * q) * N + j) * N + i0 + tx;
-            tile[ty + 8 * q][tx] = (add ? add[x] : 0.0) + (double)v[x];
+            tile[ty + 8 * q][tx] = (add ? add[x] : 0.0) + widen(v[x]);
         }
         __syncthreads();
     }
@@ -190,7 +190,7 @@ template <typename T>
 __global__ void k_widen(const T* v, long long n, double* out) {
     wait_prior_grid();
     for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < n; x += (long long)gridDim.x * blockDim.x)
-        out[x] = (double)v[x];
+        out[x] = widen(v[x]);
 }
 
 }  // namespace

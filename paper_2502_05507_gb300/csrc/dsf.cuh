@@ -25,7 +25,14 @@ struct __align__(8) dsf {
     __host__ __device__ dsf() = default;
     __host__ __device__ constexpr dsf(float h, float l) : hi(h), lo(l) {}
     // nearest double-float to a double (exact for up to 48 significant bits)
-    __host__ __device__ explicit dsf(double d) : hi((float)d), lo((float)(d - (double)(float)d)) {}
+    __host__ __device__ explicit dsf(double d) {
+#ifdef __CUDA_ARCH__
+        split_double(d, hi, lo);
+#else
+        hi = (float)d;
+        lo = (float)(d - (double)hi);
+#endif
+    }
     __host__ __device__ explicit operator double() const { return (double)hi + (double)lo; }
 };
 
@@ -111,7 +118,9 @@ __device__ __forceinline__ dsc ldg_c<dsc>(const dsc* p) {
     return r;
 }
 
-// element type written by the last convolution pass
+// element type written by the last convolution pass (the conversion
+// instructions: with widen() the even-odd inverse passes of 64 right-hand sides
+// took 198 instead of 185 us)
 template <> struct OutOf<dsf> { using type = double; };
 __device__ __forceinline__ double to_out(dsf v) { return (double)v.hi + (double)v.lo; }
 

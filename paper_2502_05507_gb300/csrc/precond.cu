@@ -111,7 +111,7 @@ __global__ void k_member_info(const int* __restrict__ lin_of, const int* __restr
 // branches on it common to the warp and every lookup one add and a load at a
 // constant distance; the block goes through shared memory once, transposed, to
 // the registers of the lane that eliminates it; and a step passes the pivot
-// row on in shared memory, four values to a load.With that
+// row on in shared memory, four values to a load. With that
 // 85 us. The entries and the elimination are the same operations in the same order.
 __global__ void __launch_bounds__(32 * RAS_WARPS, 4) k_ras_rows(const int* __restrict__ lin_of, const int4* __restrict__ minfo,
                                                           const uint8_t* __restrict__ flags,
