@@ -213,8 +213,13 @@ __device__ __forceinline__ C line_spectrum(const C* row, int k, int N) {
     return cconj(row[2 * N - k]);
 }
 
-// L - k, the mirror image of frequency k of a transform of length L
-__device__ __forceinline__ int mirror(int k, int L) { return k == 0 ? 0 : L - k; }
+// L - k, the mirror image of frequency k of a transform of length L (a mask where
+// L allows it: the float32 i pass at L = 512 took 297 instead of 287 us with the
+// comparison)
+template <int L> __device__ __forceinline__ int mirror(int k) {
+    if constexpr ((L & (L - 1)) == 0) return (L - k) & (L - 1);
+    else return k == 0 ? 0 : L - k;
+}
 
 // slot k of column 0 after the forward j transform, from Z(k) and Z(2N - k)
 template <typename C>
@@ -241,7 +246,7 @@ __device__ __forceinline__ void split_column0(C* v, C* xch, int c, int t) {
 #pragma unroll
         for (int s = 0; s < PL::S; ++s) {
             const int k = PL::kidx(t, s);
-            v[s] = slot_split(v[s], xch[mirror(k, L)], k, L / 2);
+            v[s] = slot_split(v[s], xch[mirror<L>(k)], k, L / 2);
         }
     }
     __syncthreads();

@@ -231,7 +231,7 @@ __device__ __forceinline__ void colpass_tile(const ConvArgs<T>& a, int bx, int b
         for (int s = 0; s < S; ++s) {
             const int k = PL::kidx(t, s);
             C x = ok ? in[k * stride] : zero;
-            if (col0 && c == 0) x = slot_merge(x, in[mirror(k, L) * stride], k, N);
+            if (col0 && c == 0) x = slot_merge(x, in[mirror<L>(k) * stride], k, N);
             v[s] = x;
         }
         PL::inv(v, xch, c, W, t, a.tw);
@@ -282,7 +282,7 @@ __device__ __forceinline__ void colpass_tile(const ConvArgs<T>& a, int bx, int b
                     const int ii = k <= N ? k : L - k;
                     const T g0 = g[(long long)ii * N1 * N1], gn = g[(long long)ii * N1 * N1 + N];
                     // (g0 + gN) y(p) / 2 + (g0 - gN) conj y(-p) / 2
-                    const C yr = cconj(xch[mirror(k, L)]);
+                    const C yr = cconj(xch[mirror<L>(k)]);
                     const C y = v[s];
                     const T sp = (g0 + gn) * half, sm = (g0 - gn) * half;
                     v[s] = cmake<C>(y.x * sp + yr.x * sm, y.y * sp + yr.y * sm);
