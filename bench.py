@@ -152,7 +152,18 @@ def kernel_model(n, pb, n_gm, npl=None, nb=1):
     F = 5.0 * L * math.log2(L)
     src = 8 * n_gm + 4 * (npl * n + 1)
     plane_f = (npl * n / 2) * F + npl * n * F
+    # the even-odd schedule on the window of nt = 3 n / 4 nodes that the bodies
+    # of these workloads fit (n >= 64): rows of nt lines for the npl planes, the
+    # m x m products of both halves (m = npl / 2) for the four real vectors of
+    # nt frequency pairs per k column, two flops each
+    nt = 3 * n // 4 if n >= 64 else n
+    Fw = 5.0 * 2 * nt * math.log2(2 * nt)
+    Aw = npl * nt * nt * c
+    m = (npl + 1) // 2
     return {
+        "conv_eo_fwd": (Aw + src, (npl * nt / 2) * Fw),
+        "conv_eo_mid": (2 * Aw + npl * (nt + 1) ** 2 * pb / nb, 2 * npl * nt * Fw + 2 * m * m * 8.0 * nt * nt),
+        "conv_eo_inv": (Aw + npl * nt * nt * pb, (npl * nt / 2) * Fw),
         "conv_kfwd": (A + src, (npl * n / 2) * F),
         "conv_jfwd": (A + B, npl * n * F),
         # i pass: reads and writes the rows of the transformed planes
@@ -193,8 +204,10 @@ DF64_OPS_PER_FLOP = 7.0
 # is dropped from this table (its traffic is then reported as null). Keyed
 # by (kernel, N, right-hand sides per launch).
 NCU_TRAFFIC = {
-    # conv_i_narrow_batched32_torus_N128.md: 494.8 MB per 32-right-hand-side
-    # launch, scaled by 2 less one extra read of the 8.6 MB spectrum octant
+    # the i pass on 32 planes of the whole grid, 494.8 MB per 32-right-hand-side
+    # launch, scaled by 2 less one extra read of the 8.6 MB spectrum octant (its
+    # transform form; the default workload's even-odd kernels keep these rows in
+    # shared memory and move little DRAM: conv_eo_batched16_torus_N128.md)
     ("conv_i.f32", 128, 64): 2 * 494.8e6 - 8.59e6,
 }
 
@@ -252,13 +265,15 @@ def kernel_table(prof, top=16):
 
 
 def apply_summary(prof, n, npl, nb, hbm, suffix=".f32"):
-    """Whole float32 apply: the minimum bytes of apply_bytes_min over the
-    summed time per apply of the passes that ran (either schedule)."""
+    """Whole float32 apply: the minimum bytes of apply_bytes_min (an apply
+    whose padded field goes through memory on the whole grid: the even-odd
+    schedule on a window moves less) over the summed time per apply of the
+    passes that ran (any schedule)."""
     names = [k for k in prof if k.startswith("conv_") and k.endswith(suffix)]
-    ikey = "conv_i" + suffix
-    if ikey not in prof:
+    # launches of the pass along i: one per apply, in either form
+    napp = sum(prof[k + suffix][1] for k in ("conv_i", "conv_eo_mid") if k + suffix in prof)
+    if napp == 0:
         return None
-    napp = prof[ikey][1]
     t_apply = sum(prof[k][0] for k in names) / napp / 1000.0
     nbytes = apply_bytes_min(n, 4, npl, nb) * nb
     return {"us_per_apply": t_apply * 1e6, "rhs_per_apply": nb, "passes": sorted(k.split(".")[0] for k in names),

@@ -160,7 +160,12 @@ long long bae_launch_count(void);
  * at once, striding over the tiles of every right-hand side of the batch.
  * All compute the same convolution (Section 3.2, the
  * discrete potentials as lattice sums); they differ in rounding order only.
- * A schedule the size cannot run falls back to BAE_SCHED_PASSES. Overrides
+ * A schedule the size cannot run falls back to BAE_SCHED_PASSES. Left to
+ * itself (BAE_SCHED_AUTO) an apply whose planes it covers takes the even-odd
+ * schedule (three kernels, no timing), and an apply inside a solve or
+ * bae_boundary_apply runs on a window of 3N/4 nodes per axis where sources and
+ * read-back nodes fit it (N >= 64); a forced schedule transforms the whole
+ * grid. Overrides
  * the BAE_CONV_PLANE environment variable (0, 1, 2 or 3: the same values).
  * Returns BAE_ERR_INVALID_ARG for any other value. Not part of the method:
  * a performance control. */
@@ -342,9 +347,8 @@ int bae_boundary_apply(bae_problem* prob, int precision, const double* q, double
  *    bae_problem_create, which does allocate, at set-up.
  *  - The first call on a device looks up the device address of the array
  *    (cudaGetSymbolAddress); make that first call before any stream capture.
- *  - The call never times convolution schedules: it uses the schedule an
- *    earlier apply of the same precision and N (one right-hand side) chose,
- *    or bae_set_conv_schedule's, else the plane-fused default.
+ *  - The call never times convolution schedules: it uses
+ *    bae_set_conv_schedule's, else the even-odd schedule.
  *  - Every call uses the same array and leaves its contents behind; nothing
  *    in it needs clearing, since each call writes every element it reads.
  *    Calls whose GPU work overlaps in time (several host threads, several

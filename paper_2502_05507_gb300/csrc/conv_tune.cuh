@@ -15,7 +15,8 @@ namespace bae {
 // N, batch size) outside a graph capture times every runnable schedule on
 // the real data and keeps the fastest; the choices persist in the JSON file
 // named by BAE_TUNE_FILE if set. BAE_CONV_PLANE=0/1/2/3 forces a schedule
-// (the Sched values).
+// (the Sched values). An apply that the even-odd schedule covers (conv_eo.cuh)
+// takes it unless a schedule is forced, and is not timed here.
 
 // SCHED_PASSES_ALT: the five passes with the variant-1 launch geometry
 // (float32: half-width column blocks at N = 128, the three-level transform
