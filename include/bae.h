@@ -71,7 +71,11 @@ typedef struct bae_ctx bae_ctx;
 typedef struct bae_problem bae_problem;
 
 typedef struct bae_options {
-    double tol;          /* relative residual ||b - A q|| / ||b||, default 1e-10 */
+    double tol;          /* relative residual ||b - A q|| / ||b||, default 1e-10.
+                            BAE_MIXED with tol >= 1e-11: a right-hand side that
+                            ends a refinement step between tol / 2 and tol is
+                            taken one step further (within max_refine and
+                            max_iter), and keeps the better of the two       */
     int    max_iter;     /* total GMRES iterations (all cycles), default 500    */
     int    restart;      /* GMRES restart length, 1..1024, default 200          */
     int    precision;    /* BAE_FP64 (every apply native float64), BAE_DF64

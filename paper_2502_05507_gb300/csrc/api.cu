@@ -172,12 +172,13 @@ struct Workspace {
     Grow<unsigned long long> arnBar;
     Grow<double> in_f, in_g, out_q, out_u;    // staging of host arguments
     Grow<double> qpre, zpre;                  // M^{-1} y of the preconditioned inner solves
+    Grow<double> qmet;                        // densities that reached tol, beside a further refinement step
     Grow<float> arnV32, arnZ32;               // float32 copies of the newest basis vector and its M^{-1}
     Grow<double> ydir64, bprime;              // direct formulation: operator rows, [g; 0]
     Grow<float> ydir32;
     void set_stream(cudaStream_t st) {
         Grow<double>* ds[] = {&v64, &up, &vstage, &V, &w, &partial, &h, &hsave, &x, &r, &bvec, &tmp,
-                              &qstage, &n2, &in_f, &in_g, &out_q, &out_u, &qpre, &zpre, &ydir64, &bprime};
+                              &qstage, &n2, &in_f, &in_g, &out_q, &out_u, &qpre, &zpre, &qmet, &ydir64, &bprime};
         for (auto* d : ds) d->st = st;
         Grow<double>* ds2[] = {&arnH, &arnHu, &arnCS, &arnG, &arnY, &arnScal};
         for (auto* d : ds2) d->st = st;
@@ -1237,16 +1238,24 @@ int solve_impl(bae_problem* P, int nb, const double* f, const double* g, const b
         for (int b = 0; b < nb; ++b) relres[b] = bn2[b] > 0 ? 1.0 : 0.0;
         int iters_left = o.max_iter;
         StepGraph step_graph;   // the inner solves' captured step, shared by the refinement steps
-        // A residual between half of tol and tol is taken one step further (tolerances
-        // well above what the float64-accurate residual resolves): whether the
-        // rounding of the float32 applies lands at 0.9 or 1.1 tol decided between
-        // two steps and three, with solutions up to 50 times apart in error. 3 of
-        // 160 solves (N = 32 to 256, every layer, tol 1e-10) take it.
-        const double stop = o.tol >= 1e-11 ? 0.5 * o.tol : o.tol;
+        // A right-hand side whose residual lies between half of tol and tol is taken
+        // one step further, once (tolerances well above what the float64-accurate
+        // residual resolves): whether the rounding of the float32 applies lands at 0.9
+        // or 1.1 tol decided between two steps and three, with solutions up to 50
+        // times apart in error. 3 of 160 solves (N = 32 to 256, every layer, tol
+        // 1e-10) take it. Where the step does not lower the residual, which lies at
+        // the rounding of the float64-accurate applies then, its q is put back.
+        const double half_tol = 0.5 * o.tol;
+        const bool further = o.tol >= 1e-11;
+        std::vector<char> taken(nb, 0);   // has had its step below tol
         for (int step = 0; step < std::max(1, o.max_refine); ++step) {
-            std::vector<int> act;
-            for (int b = 0; b < nb; ++b)
-                if (relres[b] > stop && bn2[b] > 0) act.push_back(b);
+            std::vector<int> act, met;   // met: those of act that have reached tol
+            for (int b = 0; b < nb; ++b) {
+                if (!(bn2[b] > 0)) continue;
+                const bool again = relres[b] <= o.tol && relres[b] > half_tol && further && !taken[b];
+                if (relres[b] > o.tol || again) act.push_back(b);
+                if (again) met.push_back(b);
+            }
             if (act.empty() || iters_left <= 0) break;
             // every refinement step (precond 1) or the steps after the first
             // (precond 2)
@@ -1272,6 +1281,12 @@ int solve_impl(bae_problem* P, int nb, const double* f, const double* g, const b
             gmres(P, BAE_FP32, nb, act, res, d, true, Si, iters_left, o.restart, applies, o.use_graphs != 0, use_pre,
                   &step_graph);
             if (use_pre) precond_apply(P->pre, d, n, nullptr, 0, dq, n, nb, nullptr, st);
+            // the q that reached tol, kept beside the step
+            const std::vector<double> rel_met = relres;
+            double* q_met = met.empty() ? nullptr : P->ws().qmet.need((long long)nb * n);
+            for (int b : met)
+                BAE_CUDA(cudaMemcpyAsync(q_met + (long long)b * n, q + (long long)b * n, (size_t)n * sizeof(double),
+                                         cudaMemcpyDeviceToDevice, st));
             int used = 0;
             for (int b : act) {
                 st_local[b].iterations += Si[b].iterations;
@@ -1284,6 +1299,15 @@ int solve_impl(bae_problem* P, int nb, const double* f, const double* g, const b
             kr_add(use_pre ? dq : d, d_a, (int)act.size(), n, q, st);
             for (int b : act) st_local[b].applies_fp32 += applies[b];
             true_residual();
+            bool back = false;
+            for (int b : met) {
+                taken[b] = 1;
+                if (relres[b] < rel_met[b]) continue;
+                BAE_CUDA(cudaMemcpyAsync(q + (long long)b * n, q_met + (long long)b * n, (size_t)n * sizeof(double),
+                                         cudaMemcpyDeviceToDevice, st));
+                back = true;
+            }
+            if (back) true_residual();
         }
         if (!v_last) true_residual();
     }
