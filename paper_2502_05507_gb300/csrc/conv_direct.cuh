@@ -45,7 +45,9 @@ template <typename T> struct DirTile {
 };
 
 // acc += p x; for double-float the product's error, its cross terms and the
-// sum's error go to the low part (12 float operations), normalised at the end
+// sum's error go to the low part (12 float operations). The low part's own
+// rounding grows with it, so dir_norm puts the sum in order after every block
+// of TJ terms.
 __device__ __forceinline__ void dir_fma(float& acc, float p, float x) { acc = __fmaf_rn(p, x, acc); }
 __device__ __forceinline__ void dir_fma(double& acc, double p, double x) { acc = __fma_rn(p, x, acc); }
 __device__ __forceinline__ void dir_fma(dsf& acc, dsf p, dsf x) {
@@ -56,6 +58,9 @@ __device__ __forceinline__ void dir_fma(dsf& acc, dsf p, dsf x) {
     const dsf s = two_sum(acc.hi, h);
     acc = dsf(s.hi, __fadd_rn(acc.lo, __fadd_rn(s.lo, e)));
 }
+__device__ __forceinline__ float dir_norm(float a) { return a; }
+__device__ __forceinline__ double dir_norm(double a) { return a; }
+__device__ __forceinline__ dsf dir_norm(dsf a) { return fast_two_sum(a.hi, a.lo); }
 __device__ __forceinline__ float dir_half(float a) { return 0.5f * a; }
 __device__ __forceinline__ double dir_half(double a) { return 0.5 * a; }
 __device__ __forceinline__ dsf dir_half(dsf a) { return dsf(0.5f * a.hi, 0.5f * a.lo); }
@@ -130,6 +135,13 @@ __device__ __forceinline__ void direct_rows_product(const typename DirRow<T, NV>
                     }
                 }
             }
+#pragma unroll
+            for (int i = 0; i < TI; ++i)
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    ae[i][v] = dir_norm(ae[i][v]);
+                    ao[i][v] = dir_norm(ao[i][v]);
+                }
         }
 #pragma unroll
         for (int i = 0; i < TI; ++i) {

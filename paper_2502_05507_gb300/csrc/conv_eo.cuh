@@ -272,10 +272,6 @@ __global__ void __launch_bounds__(EoGeo<T, L>::KT) k_eo_inv(ConvArgs<T> a, int n
 }
 
 // ------------------------------------------------- middle pass (j, i, j^-1)
-__device__ __forceinline__ float dir_norm(float a) { return a; }
-__device__ __forceinline__ double dir_norm(double a) { return a; }
-__device__ __forceinline__ dsf dir_norm(dsf a) { return fast_two_sum(a.hi, a.lo); }
-
 // entry g(|i-j|) +- g(n-1-i-j): one fused multiply-add with the sign, or the
 // sum with a value flipped when it was loaded (double-float)
 template <typename T>
@@ -335,6 +331,10 @@ __device__ __forceinline__ void eo_product(T (&acc)[DirTile<T>::TI][4], const T*
                 }
             }
         }
+#pragma unroll
+        for (int i = 0; i < TI; ++i)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) acc[i][v] = dir_norm(acc[i][v]);
     };
     const int full = m / TJ;
     for (int jb = 0; jb < full; ++jb) block(jb, TJ, std::true_type{});
@@ -484,8 +484,8 @@ __global__ void __launch_bounds__(MAXW * 32, MINB) k_eo_mid(ConvArgs<T> a, EoSha
                 for (int i = 0; i < TI; ++i) {
                     const int r = TI * ib + i;
                     if (r < m) {   // the middle frequency is its own image: the same value twice
-                        pa[r * XS] = cmake<C>(dir_norm(acc[i][0]), dir_norm(acc[i][1]));
-                        pb[r * XS] = cmake<C>(dir_norm(acc[i][2]), dir_norm(acc[i][3]));
+                        pa[r * XS] = cmake<C>(acc[i][0], acc[i][1]);
+                        pb[r * XS] = cmake<C>(acc[i][2], acc[i][3]);
                     }
                 }
             }
