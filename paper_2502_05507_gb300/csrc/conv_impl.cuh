@@ -192,7 +192,11 @@ __global__ void __launch_bounds__(Geo<T, L, V>::KT, Geo<T, L, V>::MINB_KF) k_kpa
 // ----------------------------------------------------- column passes (j, i)
 enum ColMode { COL_FWD_J = 0, COL_CONV_I = 1, COL_INV_J = 2 };
 
-template <typename T, int L, int MODE, bool BOX, int V>
+// NARROW (the i pass of at most L / 4 planes, !BOX): the pencil is transformed
+// shifted so that plane p0 is row 0. Its rows are the first quarter, so the first
+// DFT drops the zero slots and the last one forms only those stored back; a circular
+// convolution commutes with the shift.
+template <typename T, int L, int MODE, bool BOX, int V, bool NARROW>
 __device__ __forceinline__ void colpass_tile(const ConvArgs<T>& a, int bx, int by, int bz) {
     using C = cplx_t<T>;
     using G = Geo<T, L, V>;
@@ -225,7 +229,15 @@ __device__ __forceinline__ void colpass_tile(const ConvArgs<T>& a, int bx, int b
 
     C v[S];
     const C zero = cmake<C>((T)0, (T)0);
-    if (MODE == COL_INV_J) {
+    static_assert(!NARROW || (MODE == COL_CONV_I && !BOX), "i pass only");
+    if constexpr (NARROW) {
+        const int np = a.plane_hi() - a.plane_lo();
+        in += a.plane_lo() * stride;
+        out += a.plane_lo() * stride;
+#pragma unroll
+        for (int m = 0; m < S; ++m) v[m] = (m < S / 4 && ok && t + TH * m < np) ? in[(t + TH * m) * stride] : zero;
+        PL::template fwd<2>(v, xch, c, W, t, a.tw);
+    } else if (MODE == COL_INV_J) {
         // k-layout load of all L rows (column 0: merge slots k and L - k)
 #pragma unroll
         for (int s = 0; s < S; ++s) {
@@ -314,8 +326,13 @@ __device__ __forceinline__ void colpass_tile(const ConvArgs<T>& a, int bx, int b
         }
         PL::inv(v, xch, c, W, t, a.tw);
     }
-    // n-layout store of the first N rows
-    if (ok) {
+    // n-layout store of the first N rows (NARROW: of the planes, from p0)
+    if constexpr (NARROW) {
+        const int np = a.plane_hi() - a.plane_lo();
+#pragma unroll
+        for (int m = 0; m < S / 4; ++m)
+            if (ok && t + TH * m < np) out[(t + TH * m) * stride] = v[m];
+    } else if (ok) {
 #pragma unroll
         for (int m = 0; m < S; ++m) {
             const int n = t + TH * m;
@@ -329,7 +346,7 @@ __device__ __forceinline__ void colpass_tile(const ConvArgs<T>& a, int bx, int b
 // tiles (column block, line, right-hand side), column blocks fastest:
 // strided over a grid of resident CTAs (PERSIST) or one per CTA of the grid
 // (column blocks, lines, right-hand sides)
-template <typename T, int L, int MODE, bool BOX = false, int V = 0, bool PERSIST = false>
+template <typename T, int L, int MODE, bool BOX = false, int V = 0, bool PERSIST = false, bool NARROW = false>
 __global__ void __launch_bounds__(Geo<T, L, V>::CT, Geo<T, L, V>::minb_col(MODE)) k_colpass(ConvArgs<T> a) {
     wait_prior_grid();   // results of the previous kernel on the stream
     if constexpr (PERSIST) {
@@ -340,11 +357,11 @@ __global__ void __launch_bounds__(Geo<T, L, V>::CT, Geo<T, L, V>::minb_col(MODE)
         const long long ntiles = per_b * a.nbatch;
         for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
             const long long rem = tile % per_b;
-            colpass_tile<T, L, MODE, BOX, V>(a, (int)(rem % ncb), (int)(rem / ncb), (int)(tile / per_b));
+            colpass_tile<T, L, MODE, BOX, V, NARROW>(a, (int)(rem % ncb), (int)(rem / ncb), (int)(tile / per_b));
             __syncthreads();   // the next tile reuses the shared memory
         }
     } else {
-        colpass_tile<T, L, MODE, BOX, V>(a, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z);
+        colpass_tile<T, L, MODE, BOX, V, NARROW>(a, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z);
     }
 }
 
@@ -608,6 +625,15 @@ __global__ void __launch_bounds__(512) k_plane_inv(ConvArgs<T> a) {
     }
 }
 
+// The narrow i pass: double-float at L = 512 (three-level plan, 64 threads per
+// line), where the direct sum ends before L / 4 = 128 planes. 110 to 118 planes,
+// the transform over all rows / over two of the four slots: 1060 / 989 us, the
+// operator 1416 / 1398 us; the direct sum would take the operator to 1473 us at 108
+// planes (1382 both at 104).
+template <typename T, int L> struct NarrowI {
+    static constexpr bool value = std::is_same<T, dsf>::value && L == 512;
+};
+
 template <typename T, int L>
 void configure_passes() {
     using C = cplx_t<T>;
@@ -622,6 +648,10 @@ void configure_passes() {
         set(k_kpass_inv<T, L>, smem_k);
         set(k_colpass<T, L, COL_FWD_J>, smem_c);
         set(k_colpass<T, L, COL_CONV_I>, smem_c);
+        if constexpr (NarrowI<T, L>::value) {
+            set(k_colpass<T, L, COL_CONV_I, false, 0, false, true>, smem_c);
+            set(k_colpass<T, L, COL_CONV_I, false, 0, true, true>, smem_c);
+        }
         set(k_colpass<T, L, COL_INV_J>, smem_c);
         return true;
     }();
@@ -712,7 +742,7 @@ dim3 persist_grid(long long ntiles, K kernel, int threads, size_t smem) {
 }
 
 // the i pass (not the finite box): the direct sum over the planes where it
-// can be. The choice depends on the element type, N and the plane range only,
+// can be, the narrow transform where it exists and covers them. The choice depends on the element type, N and the plane range only,
 // so that every schedule and batch size takes the same one (bit-identical
 // results).
 template <typename T, int L, int V, bool PERSIST = false>
@@ -720,6 +750,16 @@ void launch_conv_i(const ConvArgs<T>& a, dim3 grid, size_t smem, cudaStream_t st
     if (a.gmix && a.plane_hi() - a.plane_lo() <= direct_i_limit<T>(L / 2)) {
         launch_direct_i<T>(a, st);
         return;
+    }
+    if constexpr (NarrowI<T, L>::value) {
+        if (a.plane_hi() - a.plane_lo() <= L / 4) {
+            auto k = k_colpass<T, L, COL_CONV_I, false, V, PERSIST, true>;
+            if constexpr (PERSIST)
+                grid = persist_grid((long long)ceil_div(L / 2, Geo<T, L, V>::W) * L * a.nbatch, k, Geo<T, L, V>::CT, smem);
+            BAE_LAUNCH(kname<T>("conv_i.f32", "conv_i.f64", "conv_i.df64"), st,
+                       launch_pdl(k, grid, Geo<T, L, V>::CT, smem, st, a));
+            return;
+        }
     }
     BAE_LAUNCH(kname<T>("conv_i.f32", "conv_i.f64", "conv_i.df64"), st,
                launch_pdl(k_colpass<T, L, COL_CONV_I, false, V, PERSIST>, grid, Geo<T, L, V>::CT, smem, st, a));

@@ -238,6 +238,14 @@ __device__ __forceinline__ void rdft_zhi(C* v) {
     }
 }
 
+// the same with v[R/4..R) zero, R = 8
+template <int R, bool INV, typename C>
+__device__ __forceinline__ void rdft_zquarter(C* v) {
+    static_assert(R == 8, "two values");
+    const C e[4] = {v[0], v[0], v[0], v[0]}, o[4] = {v[1], v[1], v[1], v[1]};
+    Bflies<R, INV, C, 0>::run(e, o, v);
+}
+
 // The barrier around an exchange: the CTA's, or (WARP) the warp's where all
 // threads of a line are in one warp.
 template <bool WARP>
@@ -365,9 +373,11 @@ struct Plan3_512 {
     __device__ __forceinline__ static int pos(int p) { return p + (p >> 6); }
 
     // (the threads of a line are two warps: the barriers are the CTA's)
-    template <bool ZHI, bool = false, typename C>
+    // Z: 1 the upper half of the input is zero, 2 its upper three quarters
+    template <int Z, bool = false, typename C>
     __device__ __forceinline__ static void fwd(C* v, C* xch, int base, int es, int t, const C* __restrict__ tw) {
-        if constexpr (ZHI) rdft_zhi<8, false>(v);       // v[k3]
+        if constexpr (Z == 2) rdft_zquarter<8, false>(v);   // v[k3]
+        else if constexpr (Z == 1) rdft_zhi<8, false>(v);
         else rdft<8, false>(v);
 #pragma unroll
         for (int k3 = 1; k3 < 8; ++k3) v[k3] = cmul(v[k3], ldg_c(tw + t * k3));
