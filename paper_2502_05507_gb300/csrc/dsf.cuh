@@ -107,6 +107,7 @@ __device__ __forceinline__ dsc cmulc(dsc a, dsc b) { return dsc{dot2(a.x, b.x, a
 __device__ __forceinline__ dsc chalf(dsc a) {
     return dsc{dsf(0.5f * a.x.hi, 0.5f * a.x.lo), dsf(0.5f * a.y.hi, 0.5f * a.y.lo)};
 }
+__device__ __forceinline__ dsc cnorm(dsc a) { return dsc{fast_two_sum(a.x.hi, a.x.lo), fast_two_sum(a.y.hi, a.y.lo)}; }
 __device__ __forceinline__ dsc crot(dsc x, dsf c, dsf s) { return dsc{dot2(x.x, c, -x.y, s), dot2(x.x, s, x.y, c)}; }
 
 template <>
