@@ -132,31 +132,39 @@ struct Grow {
     ~Grow() { release(); }
 };
 
-// One LGF spectrum, shared by every problem (and every context of a
-// server) with the same (N, s); plain cudaMalloc so that it outlives the
-// stream that built it.
-struct Spectrum {
-    int N = 0;
-    double s = 0.0;
-    double* g64 = nullptr;
-    float* g32 = nullptr;
-    dsf* gds = nullptr;
-    // the mixed spectrum (offset along the first axis, frequency along the
-    // other two) of the direct i pass; none for the finite box
-    double* m64 = nullptr;
-    float* m32 = nullptr;
-    dsf* mds = nullptr;
-    double* near = nullptr;   // G_s on the offsets below NEAR_TN (preconditioner blocks)
-    size_t bytes = 0;
-    ~Spectrum() {
-        if (g64) cudaFree(g64);
-        if (g32) cudaFree(g32);
-        if (gds) cudaFree(gds);
-        if (m64) cudaFree(m64);
-        if (m32) cudaFree(m32);
-        if (mds) cudaFree(mds);
-        if (near) cudaFree(near);
+// Forms of an LGF spectrum, a bit each: the octant (frequency along every
+// axis) and the mixed form (offset along the first axis, frequency along the
+// other two: the even-odd schedule and the direct i pass), by element type, and
+// G_s on the offsets below NEAR_TN (preconditioner blocks).
+enum SpecForm : unsigned { OCT_F64 = 1, OCT_F32 = 2, OCT_DS = 4, OCT_ALL = 7, MIX_F64 = 8, MIX_F32 = 16, MIX_DS = 32,
+                           MIX_ALL = 56, NEAR_TAB_F64 = 64, SPEC_FORMS = 7 };
+template <typename T>
+constexpr unsigned oct_form() {
+    return std::is_same<T, dsf>::value ? OCT_DS : (sizeof(T) == 8 ? OCT_F64 : OCT_F32);
+}
+template <typename T>
+constexpr unsigned mix_form() { return oct_form<T>() << 3; }
+
+// One array, plain cudaMalloc so that it outlives the stream that built it
+struct SpecArray {
+    void* p = nullptr;
+    explicit SpecArray(size_t bytes) {
+        alloc_check(bytes);
+        BAE_CUDA(cudaMalloc(&p, bytes));
     }
+    ~SpecArray() { cudaFree(p); }
+    SpecArray(const SpecArray&) = delete;
+    SpecArray& operator=(const SpecArray&) = delete;
+};
+
+// One LGF spectrum, its arrays shared by every problem (and every context of
+// a server) with the same (N, s). A holder sees the forms it asked for, whatever
+// others the cache has: the forms select the pass of an apply.
+struct Spectrum {
+    unsigned forms = 0;
+    std::shared_ptr<SpecArray> a[SPEC_FORMS];
+    void* at(unsigned form) const { return forms & form ? a[__builtin_ctz(form)]->p : nullptr; }
+    double* near() const { return static_cast<double*>(at(NEAR_TAB_F64)); }
 };
 
 // Work space shared by every problem of a context (calls on one context
@@ -224,64 +232,41 @@ using namespace bae;
 namespace bae {
 // Spectra keyed by (N, bit pattern of s). Thread-safe: a context that needs
 // a spectrum another one is building waits for it instead of building it
-// twice. Entries live as long as the cache.
+// twice. Entries live as long as the cache and hold the forms asked for so far. A
+// form in the three types takes 20 (N + 1)^3 bytes: the octant of the grid, and for
+// the window of the pruned applies one form per type (N = 256: 0.34 + 0.14 GB,
+// where every form of both would take 0.97).
 struct SpectrumCache {
     std::mutex mu;
     std::condition_variable cv;
     // key: (N, kind, bit pattern of s); kind 0 = the free-lattice G_s, 1 =
-    // the finite-box Green's function of eq. [aux], 2 = kind 0 for a window of
-    // the grid (no near-field table)
-    std::map<std::tuple<int, int, uint64_t>, std::shared_ptr<Spectrum>> map;
-    std::set<std::tuple<int, int, uint64_t>> building;
+    // the finite-box Green's function of eq. [aux] (octant forms)
+    using Key = std::tuple<int, int, uint64_t>;
+    std::map<Key, Spectrum> map;
+    std::set<Key> building;
 
-    std::shared_ptr<Spectrum> get(int N, double s, cudaStream_t st, int kind = 0) {
+    Spectrum get(int N, double s, unsigned forms, cudaStream_t st, int kind = 0) {
         uint64_t bits;
         std::memcpy(&bits, &s, sizeof(bits));
         const auto key = std::make_tuple(N, kind, bits);
         std::unique_lock<std::mutex> lock(mu);
+        unsigned missing;
         for (;;) {
             auto it = map.find(key);
-            if (it != map.end()) return it->second;
+            missing = forms & ~(it != map.end() ? it->second.forms : 0u);
+            if (!missing) {
+                Spectrum sp = it->second;
+                sp.forms = forms;
+                return sp;
+            }
             if (!building.count(key)) break;
             cv.wait(lock);
         }
         building.insert(key);
         lock.unlock();
-        std::shared_ptr<Spectrum> sp;
+        Spectrum made;
         try {
-            sp = std::make_shared<Spectrum>();
-            sp->N = N;
-            sp->s = s;
-            const long long n3 = (long long)(N + 1) * (N + 1) * (N + 1);
-            alloc_check(n3 * sizeof(double));
-            BAE_CUDA(cudaMalloc(&sp->g64, n3 * sizeof(double)));
-            alloc_check(n3 * sizeof(float));
-            BAE_CUDA(cudaMalloc(&sp->g32, n3 * sizeof(float)));
-            alloc_check(n3 * sizeof(dsf));
-            BAE_CUDA(cudaMalloc(&sp->gds, n3 * sizeof(dsf)));
-            sp->bytes = n3 * (sizeof(double) + sizeof(float) + sizeof(dsf));
-            const double L = 2.0 * N;
-            if (kind == 1) {
-                box_spectrum(N, s, 1.0 / (L * L * L), sp->g64, sp->g32, st);
-                to_dsf(sp->g64, n3, sp->gds, st);
-            } else {
-                const long long nm = mix_size(N);
-                alloc_check(nm * sizeof(double));
-                BAE_CUDA(cudaMalloc(&sp->m64, nm * sizeof(double)));
-                BAE_CUDA(cudaMalloc(&sp->m32, nm * sizeof(float)));
-                BAE_CUDA(cudaMalloc(&sp->mds, nm * sizeof(dsf)));
-                sp->bytes += nm * (sizeof(double) + sizeof(float) + sizeof(dsf));
-                BAE_CUDA(cudaMemsetAsync(sp->m64, 0, nm * sizeof(double), st));   // the places between the rows
-                lgf_spectrum(N, s, 1.0 / (L * L * L), sp->g64, sp->g32, st, 1.0 / (L * L), sp->m64, sp->m32);
-                to_dsf(sp->m64, nm, sp->mds, st);
-                to_dsf(sp->g64, n3, sp->gds, st);
-                if (kind == 0) {
-                    alloc_check(NEAR_TAB * sizeof(double));
-                    BAE_CUDA(cudaMalloc(&sp->near, NEAR_TAB * sizeof(double)));
-                    lgf_table(NEAR_TN, s, sp->near, st);
-                }
-            }
-            BAE_CUDA(cudaStreamSynchronize(st));
+            made = build(N, s, missing, st, kind);
         } catch (...) {
             lock.lock();
             building.erase(key);
@@ -290,16 +275,53 @@ struct SpectrumCache {
         }
         lock.lock();
         building.erase(key);
-        map[key] = sp;
+        Spectrum& sp = map[key];
+        for (int f = 0; f < SPEC_FORMS; ++f)
+            if (made.forms >> f & 1u) sp.a[f] = made.a[f];
+        sp.forms |= made.forms;
+        Spectrum out = sp;
+        out.forms = forms;
         cv.notify_all();
-        return sp;
+        return out;
     }
 
-    size_t bytes() {
-        std::lock_guard<std::mutex> lock(mu);
-        size_t b = 0;
-        for (auto& kv : map) b += kv.second->bytes;
-        return b;
+private:
+    // a float64 form that only the double-float one is made from lives in `tmp`
+    static Spectrum build(int N, double s, unsigned forms, cudaStream_t st, int kind) {
+        Spectrum sp;
+        sp.forms = forms;
+        Grow<double> tmp_oct, tmp_mix;
+        tmp_oct.st = tmp_mix.st = st;
+        auto array = [&](unsigned form, size_t bytes) -> void* {
+            if (!(forms & form)) return nullptr;
+            return (sp.a[__builtin_ctz(form)] = std::make_shared<SpecArray>(bytes))->p;
+        };
+        const long long n3 = (long long)(N + 1) * (N + 1) * (N + 1), nm = mix_size(N);
+        const double L = 2.0 * N;
+        double *g64 = nullptr, *m64 = nullptr;
+        float *g32 = nullptr, *m32 = nullptr;
+        dsf *gds = nullptr, *mds = nullptr;
+        if (forms & OCT_ALL) {
+            g64 = static_cast<double*>(array(OCT_F64, n3 * sizeof(double)));
+            g32 = static_cast<float*>(array(OCT_F32, n3 * sizeof(float)));
+            gds = static_cast<dsf*>(array(OCT_DS, n3 * sizeof(dsf)));
+            if (!g64) g64 = tmp_oct.need(n3);
+        }
+        if (forms & MIX_ALL) {
+            m64 = static_cast<double*>(array(MIX_F64, nm * sizeof(double)));
+            m32 = static_cast<float*>(array(MIX_F32, nm * sizeof(float)));
+            mds = static_cast<dsf*>(array(MIX_DS, nm * sizeof(dsf)));
+            if (!m64) m64 = tmp_mix.need(nm);
+            BAE_CUDA(cudaMemsetAsync(m64, 0, nm * sizeof(double), st));   // the places between the rows
+        }
+        if (kind == 1) box_spectrum(N, s, 1.0 / (L * L * L), g64, g32, st);
+        else if (g64 || m64) lgf_spectrum(N, s, 1.0 / (L * L * L), g64, g32, st, 1.0 / (L * L), m64, m32);
+        if (gds) to_dsf(g64, n3, gds, st);
+        if (mds) to_dsf(m64, nm, mds, st);
+        if (void* near = array(NEAR_TAB_F64, NEAR_TAB * sizeof(double)))
+            lgf_table(NEAR_TN, s, static_cast<double*>(near), st);
+        BAE_CUDA(cudaStreamSynchronize(st));
+        return sp;
     }
 };
 }  // namespace bae
@@ -353,7 +375,7 @@ struct bae_ctx {
         return tw[L] = t;
     }
 
-    std::shared_ptr<Spectrum> spectrum(int N, double s, int kind = 0) { return cache->get(N, s, stream, kind); }
+    Spectrum spectrum(int N, double s, unsigned forms, int kind = 0) { return cache->get(N, s, forms, stream, kind); }
 };
 
 // The box of the pruned applies on the grid they run on (the swapped view when
@@ -372,7 +394,7 @@ struct ConvBox {
 };
 
 static ConvBox conv_box(const Geometry& g) {
-    const int N = g.N, sw = g.cv_swap;
+    const int N = g.N, sw = g.view_axis;   // cv_swap once the view is built
     const int ax1 = sw == 1 ? 0 : 1, ax2 = sw == 2 ? 0 : 2;
     ConvBox c;
     c.p0 = g.src_lo[sw];
@@ -390,14 +412,36 @@ static ConvBox conv_box(const Geometry& g) {
     return c;
 }
 
+// The forms of the spectrum that a problem's applies read. Of the grid: the
+// octant, and the mixed form of each type whose applies run on it as even-odd
+// schedule or with the direct i pass: whole-grid applies at N <= 64, and pruned ones
+// that no window takes, by the library's choice or under a forced schedule. Of the
+// window: one form per type, by the pass that its plane count takes.
+template <typename T>
+static unsigned grid_mix(int N, const ConvBox& c) {
+    const int planes = c.p1 - c.p0;
+    const bool pruned = c.nt == N && (conv_mixed<T>(N, planes, false) || conv_mixed<T>(N, planes, true));
+    return pruned || conv_mixed<T>(N, N, false) ? mix_form<T>() : 0u;
+}
+static unsigned grid_forms(int N, const ConvBox& c) {
+    return OCT_ALL | NEAR_TAB_F64 | grid_mix<double>(N, c) | grid_mix<float>(N, c) | grid_mix<dsf>(N, c);
+}
+template <typename T>
+static unsigned window_form(const ConvBox& c) {
+    return conv_mixed<T>(c.nt, c.p1 - c.p0, false) ? mix_form<T>() : oct_form<T>();
+}
+static unsigned window_forms(const ConvBox& c) {
+    return window_form<double>(c) | window_form<float>(c) | window_form<dsf>(c);
+}
+
 struct bae_problem {
     bae_ctx* ctx = nullptr;
     Geometry geo;
     Precond pre;   // right preconditioner, built on the first mixed solve that asks for it
-    std::shared_ptr<Spectrum> spec;
-    ConvBox box;                          // planes and window of the pruned applies
-    std::shared_ptr<Spectrum> spec_win;   // spectrum of the window's size, when it is smaller than the grid
-    std::shared_ptr<Spectrum> spec_box;   // finite-box spectrum, fetched by the first box apply
+    Spectrum spec;
+    ConvBox box;         // planes and window of the pruned applies
+    Spectrum spec_win;   // spectrum of the window's size, when it is smaller than the grid
+    Spectrum spec_box;   // finite-box spectrum, fetched by the first box apply
     double kappa2 = 0.0, s = 0.0;
     // direct formulation: the Arnoldi gather reads the operator rows as they
     // are (row r of the vector at index r, weight 1)
@@ -414,17 +458,17 @@ void ctx_share_cache(bae_ctx* dst, const bae_ctx* src) { dst->cache = src->cache
 void ctx_set_shared_gpu(bae_ctx* c) { c->shared_gpu = true; }
 
 bool problem_view(const bae_problem* P, ProblemView& out) {
-    if (!P || !P->spec) return false;
+    if (!P || !P->spec.forms) return false;
     out.device = P->ctx->device;
     out.N = P->geo.N;
     out.n_gm = P->geo.n_gm;
     out.n_unk = P->geo.n_unk;
     out.stream = P->ctx->stream;
     out.rec = P->geo.recipe();
-    out.ghat64 = P->spec->g64;
-    out.ghat32 = P->spec->g32;
-    out.gmix64 = P->spec->m64;
-    out.gmix32 = P->spec->m32;
+    out.ghat64 = static_cast<const double*>(P->spec.at(OCT_F64));
+    out.ghat32 = static_cast<const float*>(P->spec.at(OCT_F32));
+    out.gmix64 = static_cast<const double*>(P->spec.at(MIX_F64));
+    out.gmix32 = static_cast<const float*>(P->spec.at(MIX_F32));
     auto it = P->ctx->tw.find(2 * P->geo.N);
     if (it != P->ctx->tw.end()) {
         out.tw64 = it->second.tw64;
@@ -461,16 +505,23 @@ ConvArgs<T> conv_args(bae_problem* P, int nb, bool pruned = false, bool windowed
     a.N = a.nt = N;
     a.nbatch = nb;
     const bool view = use_view(P, pruned);
-    const Spectrum* spec = P->spec.get();
+    const Spectrum* spec = &P->spec;
     if (pruned) {
         const ConvBox& c = P->box;
         a.p0 = c.p0;
         a.p1 = c.p1;
         a.q0 = c.q0;
         a.q1 = c.q1;
-        // (a schedule set by bae_set_conv_schedule runs on the whole grid)
-        if (windowed && P->spec_win && forced_sched() < 0) {
-            spec = P->spec_win.get();
+        // (a schedule set by bae_set_conv_schedule runs on the whole grid; the
+        // form of its direct i pass is fetched by the first apply that needs it)
+        if (windowed && forced_sched() >= 0 && !(spec->forms & mix_form<T>()) && conv_mixed<T>(N, a.p1 - a.p0, true)) {
+            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+            BAE_CUDA(cudaStreamIsCapturing(P->ctx->stream, &cs));
+            if (cs == cudaStreamCaptureStatusNone)
+                P->spec = P->ctx->spectrum(N, P->s, P->spec.forms | mix_form<T>());
+        }
+        if (windowed && P->spec_win.forms && forced_sched() < 0) {
+            spec = &P->spec_win;
             a.nt = c.nt;
             a.w0 = c.w0;
             a.w1 = c.w1;
@@ -487,19 +538,11 @@ ConvArgs<T> conv_args(bae_problem* P, int nb, bool pruned = false, bool windowed
     a.A = reinterpret_cast<cplx_t<T>*>(P->ws().A.need((long long)nb * N * N * N1));
     a.B = reinterpret_cast<cplx_t<T>*>(P->ws().B.need((long long)nb * N * 2 * N * N1));
     const Twiddles& tw = P->ctx->twiddles(2 * a.nt);
-    if constexpr (std::is_same<T, dsf>::value) {
-        a.ghat = spec->gds;
-        a.gmix = spec->mds;
-        a.tw = tw.twds;
-    } else if constexpr (sizeof(T) == 8) {
-        a.ghat = reinterpret_cast<const T*>(spec->g64);
-        a.gmix = reinterpret_cast<const T*>(spec->m64);
-        a.tw = reinterpret_cast<const cplx_t<T>*>(tw.tw64);
-    } else {
-        a.ghat = reinterpret_cast<const T*>(spec->g32);
-        a.gmix = reinterpret_cast<const T*>(spec->m32);
-        a.tw = reinterpret_cast<const cplx_t<T>*>(tw.tw32);
-    }
+    a.ghat = static_cast<const T*>(spec->at(oct_form<T>()));
+    a.gmix = static_cast<const T*>(spec->at(mix_form<T>()));
+    if constexpr (std::is_same<T, dsf>::value) a.tw = tw.twds;
+    else if constexpr (sizeof(T) == 8) a.tw = reinterpret_cast<const cplx_t<T>*>(tw.tw64);
+    else a.tw = reinterpret_cast<const cplx_t<T>*>(tw.tw32);
     return a;
 }
 
@@ -542,10 +585,9 @@ out_t<T>* apply_volume(bae_problem* P, int nb, const double* f, double scale, bo
 template <typename T>
 out_t<T>* apply_box(bae_problem* P, int nb, const double* f, double scale, bool pruned) {
     static_assert(sizeof(T) == 8, "the finite-box apply is float64-accurate");
-    if (!P->spec_box) P->spec_box = P->ctx->spectrum(P->geo.N, P->s, 1);
+    if (!P->spec_box.forms) P->spec_box = P->ctx->spectrum(P->geo.N, P->s, OCT_ALL, 1);
     ConvArgs<T> a = conv_args<T>(P, nb, pruned, false);
-    if constexpr (std::is_same<T, dsf>::value) a.ghat = P->spec_box->gds;
-    else a.ghat = reinterpret_cast<const T*>(P->spec_box->g64);
+    a.ghat = static_cast<const T*>(P->spec_box.at(oct_form<T>()));
     a.mode = SRC_VOLUME;
     a.box = true;
     a.f = f;
@@ -1059,7 +1101,7 @@ int solve_impl(bae_problem* P, int nb, const double* f, const double* g, const b
     if (any_pre && !P->pre.built) {
         BAE_CUDA(cudaEventRecord(P->ctx->fork_ev, st));
         BAE_CUDA(cudaStreamWaitEvent(P->ctx->side, P->ctx->fork_ev, 0));
-        build_precond(P->geo, P->s, P->spec->near, P->pre, P->ctx->side);
+        build_precond(P->geo, P->s, P->spec.near(), P->pre, P->ctx->side);
         BAE_CUDA(cudaEventRecord(P->ctx->join_ev, P->ctx->side));
         P->pre.pending = true;
     }
@@ -1638,22 +1680,22 @@ int bae_problem_create(bae_ctx* ctx, int N, double h, const double origin[3], co
             throw;
         }
         try {
-            P->spec = ctx->spectrum(N, P->s);
+            P->box = conv_box(P->geo);
+            P->spec = ctx->spectrum(N, P->s, grid_forms(N, P->box));
             ctx->twiddles(2 * N);   // built here so that later applies allocate nothing
         // the Schwarz rows of the default (mixed, preconditioned) solve, built
         // on the side stream from here on; a solve waits for them only when it
         // uses them
         BAE_CUDA(cudaEventRecord(ctx->fork_ev, ctx->stream));
         BAE_CUDA(cudaStreamWaitEvent(ctx->side, ctx->fork_ev, 0));
-        build_precond(P->geo, P->s, P->spec->near, P->pre, ctx->side);
+        build_precond(P->geo, P->s, P->spec.near(), P->pre, ctx->side);
         BAE_CUDA(cudaEventRecord(ctx->join_ev, ctx->side));
         P->pre.pending = true;
         // beside them on the main stream (N = 128 torus: 125 us of rows beside
         // 80 us of view)
         build_geometry_view(P->geo, ctx->stream);
-        P->box = conv_box(P->geo);
         if (P->box.nt != N) {
-            P->spec_win = ctx->spectrum(P->box.nt, P->s, 2);
+            P->spec_win = ctx->spectrum(P->box.nt, P->s, window_forms(P->box));
             ctx->twiddles(2 * P->box.nt);
         }
         if (P->direct()) {

@@ -71,9 +71,10 @@ struct ConvArgs {
     cplx_t<T>* A = nullptr;
     cplx_t<T>* B = nullptr;
     const T* ghat = nullptr;      // (N+1)^3 octant, includes 1/(2N)^3
-    // the spectrum before its transform along the first axis (direct i pass):
-    // gmix[d][jj][kk], offset d < N, jj, kk <= N, includes 1/(2N)^2, at
-    // mix_index (null: the i pass is always the FFT)
+    // the spectrum before its transform along the first axis (even-odd schedule,
+    // direct i pass): gmix[d][jj][kk], offset d < N, jj, kk <= N, includes
+    // 1/(2N)^2, at mix_index (null: the i pass is the FFT). On a window one of
+    // ghat and gmix is null, the one that its plane count does not use.
     const T* gmix = nullptr;
     const cplx_t<T>* tw = nullptr;  // twiddle tables of length 2N, then of length N (make_twiddles)
     typename OutOf<T>::type* v = nullptr;   // [nbatch][N^3] output potential
@@ -158,6 +159,12 @@ void cplane_launch(const ConvArgs<T>& a, cudaStream_t st, bool inverse);
 // graph).
 template <typename T>
 void conv_prepare(int nt);
+
+// Whether an apply of `planes` planes with transforms of length 2 nt (nt = N or a
+// window) multiplies with the mixed spectrum: the even-odd schedule or the direct
+// i pass (forced: under a schedule set by bae_set_conv_schedule).
+template <typename T>
+bool conv_mixed(int nt, int planes, bool forced);
 
 // Whether the schedule of this apply is known: fixed by its plane range or
 // by bae_set_conv_schedule, or chosen already for (element type, N, batch

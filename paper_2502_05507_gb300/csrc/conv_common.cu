@@ -220,19 +220,37 @@ void conv_apply(const ConvArgs<T>& a, cudaStream_t st) {
 }
 
 template <typename T>
+static bool eo_runs_at(const ConvArgs<T>& a) {
+    switch (a.nt) {
+        case 48: return eo_runs<T, 96>(a);
+        case 96: return eo_runs<T, 192>(a);
+        case 192: return eo_runs<T, 384>(a);
+        case 8: return eo_runs<T, 16>(a);
+        case 16: return eo_runs<T, 32>(a);
+        case 32: return eo_runs<T, 64>(a);
+        case 64: return eo_runs<T, 128>(a);
+        case 128: return eo_runs<T, 256>(a);
+        case 256: return eo_runs<T, 512>(a);
+    }
+    return false;
+}
+
+template <typename T>
+bool conv_mixed(int nt, int planes, bool forced) {
+    if (planes <= direct_i_limit<T>(nt)) return true;
+    static const T some{};
+    ConvArgs<T> a;   // what the choice looks at
+    a.N = a.nt = nt;
+    a.p1 = planes;
+    a.gmix = &some;
+    return !forced && eo_runs_at<T>(a);
+}
+
+template <typename T>
 bool conv_tuned(const ConvArgs<T>& a) {
     if (forced_sched() >= 0) return true;
     if (a.nt != a.N) return true;   // a window: no choice to make
-    bool eo = false;
-    switch (a.N) {
-        case 8: eo = eo_runs<T, 16>(a); break;
-        case 16: eo = eo_runs<T, 32>(a); break;
-        case 32: eo = eo_runs<T, 64>(a); break;
-        case 64: eo = eo_runs<T, 128>(a); break;
-        case 128: eo = eo_runs<T, 256>(a); break;
-        case 256: eo = eo_runs<T, 512>(a); break;
-    }
-    if (eo) return true;
+    if (eo_runs_at<T>(a)) return true;
     const std::string key = std::string(tname<T>()) + "/N" + std::to_string(a.N) + "/nb" + std::to_string(a.nbatch);
     return tune_lookup(key) >= 0;
 }
@@ -313,8 +331,11 @@ template void conv_apply<float>(const ConvArgs<float>&, cudaStream_t);
 template void conv_apply<double>(const ConvArgs<double>&, cudaStream_t);
 template void conv_apply<dsf>(const ConvArgs<dsf>&, cudaStream_t);
 template bool conv_tuned<float>(const ConvArgs<float>&);
+template bool conv_mixed<float>(int, int, bool);
 template bool conv_tuned<double>(const ConvArgs<double>&);
+template bool conv_mixed<double>(int, int, bool);
 template bool conv_tuned<dsf>(const ConvArgs<dsf>&);
+template bool conv_mixed<dsf>(int, int, bool);
 template void conv_prepare<float>(int);
 template void conv_prepare<double>(int);
 template void conv_prepare<dsf>(int);

@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(256) k_mixed_out(const double* __restrict__ p2
             const long long y = mix_index(N, d, j, k);
             const double v = tile[tx][r];
             m64[y] = v;
-            m32[y] = (float)v;
+            if (m32) m32[y] = (float)v;
         }
     }
 }
@@ -513,7 +513,7 @@ __global__ void k_periodic_mixed(int N, double s, double scale, double* m64, flo
         const double v = scale * (pow(lam, (double)d) + pow(lam, (double)(2 * N - d))) / (r * (1.0 - pow(lam, 2.0 * N)));
         const long long y = mix_index(N, d, j, k);
         m64[y] = v;
-        m32[y] = (float)v;
+        if (m32) m32[y] = (float)v;
     }
 }
 
@@ -527,7 +527,8 @@ void lgf_spectrum(int N, double s, double scale, double* g64, float* g32, cudaSt
     if (periodic_spectrum_applies(N, s)) {
         // the images of the (2N)-periodic Green's function are below
         // round-off: no table, no cosine transform
-        BAE_LAUNCH("k_periodic_spectrum", st,
+        if (g64)
+            BAE_LAUNCH("k_periodic_spectrum", st,
                    k_periodic_spectrum<<<(int)std::min<long long>((n3 + 255) / 256, 152LL * 16), 256, 0, st>>>(
                        N, s, scale, g64, g32));
         if (mix64)
@@ -549,8 +550,10 @@ void lgf_spectrum(int N, double s, double scale, double* g64, float* g32, cudaSt
     if (mix64)
         BAE_LAUNCH("k_mixed_out", st,
                    k_mixed_out<<<dim3(nb, nb1, (unsigned)N1), 256, 0, st>>>(c1.p, N, mix_scale, mix64, mix32));
-    BAE_LAUNCH("k_cos_fold", st, k_cos_fold<3><<<(unsigned)(N1 * nb1), 256, smem, st>>>(c1.p, c0.p, N));
-    BAE_LAUNCH("k_spectrum_out", st, k_spectrum_out<<<(int)std::min<long long>((n3 + 255) / 256, 152LL * 16), 256, 0, st>>>(c0.p, N, scale, g64, g32));
+    if (g64) {
+        BAE_LAUNCH("k_cos_fold", st, k_cos_fold<3><<<(unsigned)(N1 * nb1), 256, smem, st>>>(c1.p, c0.p, N));
+        BAE_LAUNCH("k_spectrum_out", st, k_spectrum_out<<<(int)std::min<long long>((n3 + 255) / 256, 152LL * 16), 256, 0, st>>>(c0.p, N, scale, g64, g32));
+    }
     BAE_CUDA(cudaStreamSynchronize(st));
 }
 

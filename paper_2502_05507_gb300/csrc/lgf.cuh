@@ -16,9 +16,9 @@ bool periodic_spectrum_applies(int N, double s);
 
 // Octant spectrum of G_s evenly embedded in (2N)^3 (offset N set to 0):
 // ghat[(k1 (N+1) + k2)(N+1) + k3] = sum_n Gemb(n) cos(pi k.n / N), times
-// `scale`. Writes float64 into g64 and, if g32 is not null, float32 into g32.
-// If mix64 is not null, also the mixed spectrum of the direct i pass (float64
-// and float32, mix_size values): entry (d, k2, k3), d < N, of the transform
+// `scale`. Writes float64 into g64 (null: not this one) and, if g32 is not null,
+// float32 into g32. If mix64 is not null, also the mixed spectrum of the direct i
+// pass (float64 and, if mix32 is not null, float32, mix_size values): entry (d, k2, k3), d < N, of the transform
 // along the second and third axes only, times mix_scale, at mix_index.
 void lgf_spectrum(int N, double s, double scale, double* g64, float* g32, cudaStream_t st, double mix_scale = 0.0,
                   double* mix64 = nullptr, float* mix32 = nullptr);
