@@ -144,6 +144,8 @@ void eo_configure();
 // The i pass as a direct sum (conv_direct_*.cu), in place in B.
 template <typename T>
 void launch_direct_i(const ConvArgs<T>& a, cudaStream_t st);
+template <typename T>
+void direct_configure();
 
 // The cluster plane kernels (conv_cplane_*.cu) for L where one plane of
 // k-spectra does not fit one CTA: cplane_ready sets their attributes and

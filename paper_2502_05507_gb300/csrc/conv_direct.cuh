@@ -251,6 +251,16 @@ __global__ void __launch_bounds__(DirTile<T>::MAXW * 32) k_direct_i(ConvArgs<T> 
 
 }  // namespace
 
+// Sets the kernel attribute (once per process; before any capture).
+template <typename T>
+void direct_configure() {
+    static const bool configured = []() {
+        BAE_CUDA(cudaFuncSetAttribute(k_direct_i<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        return true;
+    }();
+    (void)configured;
+}
+
 template <typename T>
 void launch_direct_i(const ConvArgs<T>& a, cudaStream_t st) {
     constexpr int TI = DirTile<T>::TI, MAXW = DirTile<T>::MAXW;
@@ -258,11 +268,7 @@ void launch_direct_i(const ConvArgs<T>& a, cudaStream_t st) {
     const int n = n0 + (n0 & 1), mb = (n / 2 + TI - 1) / TI;
     const int nreg = ceil_div((long long)N * (N + 1), 32), ncol = ceil_div(4 * N, 32);
     const size_t smem = (size_t)n * 32 * sizeof(T) + (size_t)mb * TI * 2 * 4 * 32 * sizeof(T);
-    static const bool configured = []() {
-        BAE_CUDA(cudaFuncSetAttribute(k_direct_i<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-        return true;
-    }();
-    (void)configured;
+    direct_configure<T>();
     const dim3 grid(nreg + ncol, a.nbatch);
     const int threads = 32 * (mb < MAXW ? mb : MAXW);
     BAE_LAUNCH(kname<T>("conv_i.f32", "conv_i.f64", "conv_i.df64"), st,

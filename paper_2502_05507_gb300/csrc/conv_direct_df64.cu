@@ -3,6 +3,7 @@
 
 namespace bae {
 
+template void direct_configure<dsf>();
 template void launch_direct_i<dsf>(const ConvArgs<dsf>&, cudaStream_t);
 
 }  // namespace bae

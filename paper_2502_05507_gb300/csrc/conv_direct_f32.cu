@@ -3,6 +3,7 @@
 
 namespace bae {
 
+template void direct_configure<float>();
 template void launch_direct_i<float>(const ConvArgs<float>&, cudaStream_t);
 
 }  // namespace bae

@@ -3,6 +3,7 @@
 
 namespace bae {
 
+template void direct_configure<double>();
 template void launch_direct_i<double>(const ConvArgs<double>&, cudaStream_t);
 
 }  // namespace bae

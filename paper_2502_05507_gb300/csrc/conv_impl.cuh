@@ -939,6 +939,7 @@ template <typename T, int L>
 void conv_configure() {
     if constexpr (L % 3 != 0) configure_conv<T, L>();
     else if constexpr (L >= 192) configure_passes<T, L>();
+    if (direct_i_limit<T>(L / 2) > 0) direct_configure<T>();
     eo_configure<T, L>();
 }
 
