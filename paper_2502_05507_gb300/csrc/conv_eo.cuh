@@ -543,7 +543,7 @@ void eo_configure() {
         auto set = [](auto k, size_t smem) {
             BAE_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         };
-        set(k_eo_fwd<T, L>, G::SMEM_KF);
+        if constexpr (!EoUse<T, L>::none) set(k_eo_fwd<T, L>, G::SMEM_KF);
         auto set_form = [&](auto split) {
             constexpr bool SP = decltype(split)::value;
             set(k_eo_inv<T, L, SP>, G::SMEM_KI);
@@ -578,12 +578,18 @@ void eo_configure() {
 //   float32 192 nodes, one: 82 planes 122 / 106, 108 187 / 159, 134 208 / 248
 //   double-float 192 nodes, operator, one: 82 planes 748 / 573, 96 772 / 690; 96
 //     nodes up to 64 planes (beyond, nine row blocks leave warps idle)
-//   float64: the passes with the direct i pass (96 nodes 44 planes 299 / 266,
-//     192 nodes 82 planes 2073 / 1945; the FP64 pipe bounds both).
+//   float64 96 and 192 nodes: never (EoUse; the even-odd schedule / the passes
+//     with the direct i pass: 96 nodes 44 planes 299 / 266, 192 nodes 82 planes
+//     2073 / 1945; the FP64 pipe bounds both).
+// At L = 512 (the whole grid at N = 256) every type takes it as far as its rows fit,
+// against the five passes with the direct i pass (bodies of 210 x 120 nodes, operator,
+// one; the 8-byte types fit to 96 planes):
+//   float32 44 planes 116 / 100, 92 277 / 206, 124 384 / 341
+//   double-float 16 planes 116 / 110, 44 390 / 361, 60 518 / 520, 92 1031 / 978
+//   float64 16 planes 413 / 387, 44 1498 / 1427, 92 4330 / 4064
 template <typename T, int L>
 constexpr int eo_limit() {
     if constexpr (L == 512) return 144;
-    else if constexpr (L % 3 == 0 && L >= 192 && std::is_same<T, double>::value) return 0;
     else if constexpr (L == 192 && std::is_same<T, dsf>::value) return 64;
     else if constexpr (L == 384) return sizeof(T) == 4 ? 116 : 96;
     else if constexpr (L >= 192) return sizeof(T) == 4 ? 104 : (std::is_same<T, dsf>::value ? 72 : 86);

@@ -167,10 +167,13 @@ __device__ __forceinline__ T source_value(const SrcRecipe& rec, int s, const dou
 
 // The forms of the even-odd schedule (conv_eo.cuh) per type and length: rows
 // of all 2N frequencies (not for the 16-byte elements at L = 512, whose rows
-// take 8 KB each), and rows split into the even and odd frequencies.
+// take 8 KB each), and rows split into the even and odd frequencies. None for
+// float64 on windows of 96 and 192 nodes, where the passes with the direct i pass are
+// the faster ones (eo_limit).
 template <typename T, int L> struct EoUse {
-    static constexpr bool whole = L <= 256 || (L == 512 && std::is_same<T, float>::value);
-    static constexpr bool split = (L >= 128 && L % 3 != 0) || L == 384;
+    static constexpr bool none = L % 3 == 0 && L >= 192 && std::is_same<T, double>::value;
+    static constexpr bool whole = !none && (L <= 256 || (L == 512 && std::is_same<T, float>::value));
+    static constexpr bool split = !none && ((L >= 128 && L % 3 != 0) || L == 384);
 };
 
 // ------------------------------------------------ packed Nyquist column
@@ -302,19 +305,19 @@ template <typename T, int L> struct CPlaneGeo {
 //             planes 86 / 86
 //   float64:  N = 256 122 planes 6887 / 8515; N = 128 82 planes 1057 / 1117,
 //             102 planes 1435 / 1231; N = 64 54 planes 214 / 229
-// (128 planes is also what the shared memory of the 8-byte types holds). On the
-// windows of 96 and 192 nodes, whose FFT i pass is shorter, the i pass alone:
-//   float64:  192 nodes 82 planes 1137 / 2780; 96 nodes 58 planes 145 / 328
-//   double-float: 192 nodes 44 planes 116 / 522; 96 nodes 44 planes 34 / 61
-//   float32:  192 nodes 44 planes 29 / 101
+// (128 planes is also what the shared memory of the 8-byte types holds). Float32 and
+// double-float reach it on the whole grid: float32 under a forced schedule only,
+// double-float also past the even-odd schedule's planes. On the windows of 96 and 192
+// nodes, whose FFT i pass is shorter, float64 alone does; the i pass alone: 192 nodes
+// 82 planes 1137 / 2780; 96 nodes 58 planes 145 / 328.
 template <typename T>
 inline int direct_i_limit(int N) {
     const bool f32 = std::is_same<T, float>::value, ds = std::is_same<T, dsf>::value;
     switch (N) {
         case 256: return f32 ? 132 : (ds ? 104 : 128);
-        case 192: return f32 ? 80 : (ds ? 90 : 124);
+        case 192: return f32 || ds ? 0 : 124;
         case 128: return f32 ? 68 : (ds ? 70 : 84);
-        case 96: return f32 ? 0 : (ds ? 56 : 84);
+        case 96: return f32 || ds ? 0 : 84;
         case 64: return f32 ? 0 : (ds ? 44 : 56);
         default: return 0;
     }
