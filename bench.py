@@ -137,8 +137,8 @@ def kernel_model(n, pb, n_gm, npl=None, nb=1):
     """Algorithmic (bytes, flops) per right-hand side of one launch of each
     convolution pass at grid size n, element precision pb bytes (complex =
     2 pb), when the solve transforms npl of the n planes along the axis the
-    convolution prunes (the planes that hold sources or read-back nodes, on
-    the axis with the fewest of them; all n if None) and nb right-hand sides
+    convolution prunes (the planes that hold sources, on the axis with the
+    fewest of them; all n if None) and nb right-hand sides
     share the launch (the spectrum is read once per launch). FFT flops use
     the 5 L log2 L convention per complex transform of length L = 2n; the
     spectral multiply counts 2 flops per element."""
@@ -188,6 +188,14 @@ def apply_bytes_min(n, pb, npl, nb=1):
     planes."""
     c = 2 * pb
     return 8 * c * n * n * npl + (n + 1) ** 3 * pb / nb + pb * n * n * npl
+
+
+def transformed_planes(conv_planes):
+    """(axis, count) of the planes that the pruned applies transform, from
+    Problem.conv_planes(): the range less its plane of margin on each side
+    (the bodies of these workloads stay away from the faces of the grid)."""
+    axis, lo, hi = conv_planes
+    return axis, hi - lo - 2
 
 
 FP64_PEAK_TFLOPS = 1.25   # nominal FP64 rate of GB300 (a probe measured 1.20)
@@ -343,8 +351,7 @@ def run_ours(args, rank, world, dev):
     pr0 = Problem(ctx, phi, P0.grid.h, P0.grid.origin, 0.0, "double")
     xs = np.asarray(pr0.boundary_points())
     n_gm = pr0.n_gm
-    conv_axis, plo, phi_ = pr0.conv_planes()
-    npl = phi_ - plo
+    conv_axis, npl = transformed_planes(pr0.conv_planes())
     pr0.close()
     f_h = np.stack([P.f() for P in probs])
     g_h = np.stack([P.g_at(xs) for P in probs])
@@ -501,7 +508,7 @@ def run_torus128_extra(ctx, torch, flush, hbm, hbm_kind, steps=50, warmup=3):
     pr0 = Problem(ctx, phi, P.grid.h, P.grid.origin, P.kappa2, "double")
     g = torch.from_numpy(P.g_at(np.asarray(pr0.boundary_points()))).cuda()
     n_gm = pr0.n_gm
-    conv_axis, plo, phi_ = pr0.conv_planes()
+    conv_axis, npl = transformed_planes(pr0.conv_planes())
     pr0.close()
 
     def step():
@@ -526,9 +533,9 @@ def run_torus128_extra(ctx, torch, flush, hbm, hbm_kind, steps=50, warmup=3):
             "iterations": st["iterations"], "rel_residual": st["rel_residual"],
             "max_err_vs_exact": _rel_err(u.cpu().numpy(), P.u_exact(), m),
             "kernels": kernel_table(prof, 8),
-            "roofline": roofline_for(dom, prof[dom][0], prof[dom][1], N, n_gm, hbm, hbm_kind, phi_ - plo, 1)
+            "roofline": roofline_for(dom, prof[dom][0], prof[dom][1], N, n_gm, hbm, hbm_kind, npl, 1)
             if dom else None,
-            "conv_f32_apply": apply_summary(prof, N, phi_ - plo, 1, hbm),
+            "conv_f32_apply": apply_summary(prof, N, npl, 1, hbm),
             "note": "N=128 single right-hand side: every buffer of the apply (~45 MB) stays in the 129 MB L2"}
 
 
@@ -548,7 +555,7 @@ def run_star256_table(ctx, torch, reps=3):
             pr0 = Problem(ctx, phi, P.grid.h, P.grid.origin, k2, layer)
             g = torch.from_numpy(P.g_at(np.asarray(pr0.boundary_points()))).cuda()
             n_gm = pr0.n_gm
-            conv_axis, plo, phi_ = pr0.conv_planes()
+            conv_axis, npl = transformed_planes(pr0.conv_planes())
             pr0.close()
 
             def step():
@@ -576,7 +583,7 @@ def run_star256_table(ctx, torch, reps=3):
                 torch.cuda.nvtx.range_pop()
                 prof = profile_stop()
                 row["kernels"] = kernel_table(prof, 10)
-                row["conv_f32_apply"] = apply_summary(prof, 256, phi_ - plo, 1, hbm)
+                row["conv_f32_apply"] = apply_summary(prof, 256, npl, 1, hbm)
             rows.append(row)
     return {"workload": "star r=0.6+0.1 sin5t cos3p, N=256, kappa^2 in {0,1,100}, double vs single layer, "
                         "u = exp(a.x), tol 1e-10, mixed precision", "table": rows,

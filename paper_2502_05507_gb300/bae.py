@@ -210,8 +210,10 @@ def set_conv_schedule(schedule: str = "auto"):
     """Forces the FFT convolution schedule of every potential apply in this
     process: "passes" (five kernels), "passes_alt" (the same with the second
     launch geometry), "persist" (the five as persistent kernels), "plane" (k
-    and j fused per x-plane) or "auto" (every runnable schedule timed once
-    per precision, N and batch size)."""
+    and j fused per x-plane) or "auto": the even-odd schedule (three kernels)
+    where it covers an apply's planes, on a window of 3/4 of the grid for the
+    applies of a solve that fit it; elsewhere every runnable one of the others
+    timed once per precision, N and batch size."""
     if schedule not in SCHEDULES:
         raise ValueError(f"schedule must be one of {sorted(SCHEDULES)}")
     _check(lib().bae_set_conv_schedule(SCHEDULES[schedule]))
@@ -301,14 +303,16 @@ class Problem:
             pass
 
     def plane_range(self):
-        """(lo, hi): the x-planes that hold every source and read-back node."""
+        """(lo, hi): the x-planes that hold every source and read-back node,
+        with one plane of margin on each side."""
         lo, hi = ctypes.c_int(), ctypes.c_int()
         _check(lib().bae_problem_plane_range(self._h, ctypes.byref(lo), ctypes.byref(hi)))
         return lo.value, hi.value
 
     def conv_planes(self):
-        """(axis, lo, hi): the axis (0 x, 1 y, 2 z) and plane range that the
-        convolutions inside a solve transform."""
+        """(axis, lo, hi): the axis (0 x, 1 y, 2 z) along which the convolutions
+        inside a solve skip planes, and the range of planes that hold sources,
+        with one plane of margin on each side (they transform those without)."""
         ax, lo, hi = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
         _check(lib().bae_problem_conv_planes(self._h, ctypes.byref(ax), ctypes.byref(lo), ctypes.byref(hi)))
         return ax.value, lo.value, hi.value

@@ -30,7 +30,7 @@ struct Geometry {
     double* term_coef = nullptr;
     float* term_coef32 = nullptr;  // the coefficients rounded to float32 (small integers and 6 + s)
     // x-planes [plane_lo, plane_hi) contain every source and every node the
-    // gather and the reconstruction read
+    // gather and the reconstruction read, with a plane of margin on each side
     int plane_lo = 0, plane_hi = 0;
     // the same range along each axis (0: x, 1: y, 2: z)
     int ext_lo[3] = {0, 0, 0}, ext_hi[3] = {0, 0, 0};
@@ -42,7 +42,8 @@ struct Geometry {
     // planes of its first axis only, so it runs on the grid with axis 0
     // swapped with the axis of fewest planes (cv_swap, see swap_axes; 0: no
     // swap, where x is already the narrowest, for the direct formulation and
-    // when BAE_CONV_AXIS=x). cv_lo/cv_hi is the plane range along that axis;
+    // when BAE_CONV_AXIS=x). cv_lo/cv_hi is the plane range along that axis,
+    // with its margin (the applies transform the planes of src_lo/src_hi);
     // the recipe, the flags and the gathered indices below are the
     // geometry's in the swapped layout (null when cv_swap == 0).
     int view_axis = 0;   // the axis, cv_swap once build_geometry_view has built the view

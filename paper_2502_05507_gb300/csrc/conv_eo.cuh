@@ -20,6 +20,8 @@
 //              / 2 and v(i', j) = (E - O) / 2
 // The 2N-wide rows (B of the five passes) never reach global memory: per
 // plane and line 4 complex values of A move instead of 2 of A and 8 of B.
+// (Plane counts below up to the figures of L = 512 are those of
+// bae_problem_conv_planes, two more than are transformed on a window.)
 // Measured at N = 128, 32 planes, 64 right-hand sides (five passes with the
 // direct i pass / these): float32 789 / 468 us per apply (the middle pass 317:
 // 70% of the issue slots, a fifth of HBM), double-float 3.21 / 2.77 ms (the
