@@ -208,15 +208,16 @@ DF64_OPS_PER_FLOP = 7.0
 
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum)
 # of convolution kernels, from ncu captures of the current kernels and
-# workloads (profiles/); a kernel or plane range changed since its capture
+# workloads; a kernel or plane range changed since its capture
 # is dropped from this table (its traffic is then reported as null). Keyed
 # by (kernel, N, right-hand sides per launch).
 NCU_TRAFFIC = {
-    # the i pass on 32 planes of the whole grid, 494.8 MB per 32-right-hand-side
-    # launch, scaled by 2 less one extra read of the 8.6 MB spectrum octant (its
-    # transform form; the default workload's even-odd kernels keep these rows in
-    # shared memory and move little DRAM: conv_eo_batched16_torus_N128.md)
-    ("conv_i.f32", 128, 64): 2 * 494.8e6 - 8.59e6,
+    # the direct i pass on the torus's 30 planes of the whole grid (the five passes
+    # forced; the default's even-odd kernels keep these rows in shared memory and
+    # read little but their input): 448.5 MB per launch of 32 right-hand sides, scaled
+    # by 2 less one extra read of the 30 planes' spectrum, 2.04 MB. The algorithmic
+    # bytes are 506: the last rows written stay in L2
+    ("conv_i.f32", 128, 64): 2 * 448.5e6 - 2.04e6,
 }
 
 

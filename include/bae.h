@@ -254,7 +254,9 @@ int bae_lgf_spectrum(bae_ctx* ctx, int N, double s, double* ghat);
  * -y,+z,-z with x = array axis 0, the one with the largest
  * t = phi(p)/(phi(p)-phi(m)); x* = x_p + t (x_m - x_p); row
  * t v(m) + (1-t) v(p) = g(x*), the hat basis of eq. [bc]), and fetches or
- * builds the LGF spectrum for s = kappa2 h^2.
+ * builds the LGF spectrum for s = kappa2 h^2. Spectra stay with the context
+ * (or the server): 20 (N+1)^3 bytes of device memory per (N, s), and 20 (n+1)^3
+ * more, n = 3N/4, where the applies of a solve run on a window of n nodes.
  * N: power of two in [8, 256]. h > 0. layer: BAE_LAYER_DOUBLE (a gamma- node
  * whose D_n is empty uses the single-layer column) or BAE_LAYER_SINGLE.
  * BAE_ERR_GEOMETRY if gamma- is empty or touches the box faces. */

@@ -384,8 +384,8 @@ struct bae_ctx {
 // of the grid where the box fits it (N >= 64), since a transform of length
 // 3N/2 does all that one of length 2N does for a box of 3N/4 nodes, with 3/4 of
 // the work along each of the three axes. Measured whole grid / window: star at N =
-// 256, 172 planes, float32 apply 461 / 255 us, double-float 1.67 / 1.04 ms; torus
-// at N = 128, 64 right-hand sides, float32 468 / 405 us, double-float 2.77 / 1.88
+// 256, 172 planes, float32 apply 461 / 255 us, double-float 1.67 / 1.12 ms; torus
+// at N = 128, 64 right-hand sides, float32 468 / 357 us, double-float 2.77 / 1.87
 // ms. At N = 32 the window's three short stages cost more than they save (float64
 // operator 57 / 74 us).
 struct ConvBox {

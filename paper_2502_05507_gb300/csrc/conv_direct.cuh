@@ -6,12 +6,12 @@
 //   y(i) = sum_i' g(|i - i'|; jj, kk) x(i'),   i, i' in the planes [p0, p1),
 // with g(d; jj, kk) = 1/(2N)^2 sum over the other two offsets of G_s(d, ., .)
 // times the two cosines (the LGF spectrum before its transform along the
-// first axis, Spectrum::m*). The FFT i pass transforms 2N values per pencil
+// first axis, the mixed form of the spectrum). The FFT i pass transforms 2N values per pencil
 // whatever the number n of planes; the sum costs n^2 products, needs no
 // padding, no twiddles and no exchange, and for the plane counts that the
 // pruned applies have it is the cheaper form (see direct_i_limit). Measured
 // at N = 128 with 32 planes, the FFT over the few nonzero rows before / the
-// sum: 64 right-hand sides float32 921 / 332 us, double-float 7150 / 1415 us
+// sum: 64 right-hand sides float32 921 / 332 us, double-float 7150 / 1525 us
 // per launch (bound by the float32 pipes; the float32 sum moves its 1.1 GB at
 // 3.2 TB/s); one right-hand side float64 723 / 104 us (the FP64 pipe).
 //

@@ -26,7 +26,7 @@
 // direct i pass / these): float32 789 / 468 us per apply (the middle pass 317:
 // 70% of the issue slots, a fifth of HBM), double-float 3.21 / 2.77 ms (the
 // float32 pipes). On the window of 96 nodes that torus fits: float32 357 us (the
-// middle pass 230), double-float 1.83 ms.
+// middle pass 230), double-float 1.87 ms (the middle pass 1.34).
 // Rows of A hold the lines [q0, q1) only, and column 0 packs the real kk = 0
 // and kk = N spectra as in the five passes (conv_geo.cuh).
 #pragma once
@@ -568,8 +568,8 @@ void eo_configure() {
 //     1234 / 1075, 108 1344 / 1392
 //   float32 N = 256, one: 82 planes 318 / 151, 108 351 / 212, 134 395 / 352;
 //     four: 82 1148 / 546, 134 1451 / 1283
-//   double-float N = 128, boundary operator, one: 44 planes 188 / 128, 64
-//     205 / 165, 82 234 / 290
+//   double-float N = 128, boundary operator, one: 50 planes 190 / 112, 66
+//     222 / 164, 82 234 / 290
 //   float64 N = 128, boundary operator, one: 26 planes 892 / 223, 64 1032 /
 //     623, 82 1117 / 996, 102 1231 / 1398
 // and at N <= 64 it is the faster one for every plane count (float32 N = 64:
@@ -578,8 +578,9 @@ void eo_configure() {
 //   float32 96 nodes, one: 44 planes 48.6 / 34.7, 82 57.2 / 49.5, 96 59.6 / 57.5;
 //     32: 44 planes 491 / 249, 96 859 / 854
 //   float32 192 nodes, one: 82 planes 122 / 106, 108 187 / 159, 134 208 / 248
-//   double-float 192 nodes, operator, one: 82 planes 748 / 573, 96 772 / 690; 96
-//     nodes up to 64 planes (beyond, nine row blocks leave warps idle)
+//   double-float 192 nodes, operator, one: 82 planes 748 / 573, 96 772 / 690 (both
+//     sides 4 to 7% less than now: their sums were not put in order); 96 nodes up to
+//     64 planes (beyond, nine row blocks leave warps idle)
 //   float64 96 and 192 nodes: never (EoUse; the even-odd schedule / the passes
 //     with the direct i pass: 96 nodes 44 planes 299 / 266, 192 nodes 82 planes
 //     2073 / 1945; the FP64 pipe bounds both).

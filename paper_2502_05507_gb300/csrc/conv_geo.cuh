@@ -300,9 +300,9 @@ template <typename T, int L> struct CPlaneGeo {
 // spheres, microseconds with the direct sum / with the FFT i pass):
 //   float32:  N = 256 122 planes 383 / 459, 160 planes 605 / 540; N = 128 64
 //             planes 87 / 91, 82 planes 111 / 93; N <= 64 never (latency)
-//   double-float: N = 256 82 planes 909 / 1257, 122 planes 1557 / 1392;
-//             N = 128 64 planes 174 / 205, 82 planes 282 / 234; N = 64 44
-//             planes 86 / 86
+//   double-float: N = 256 100 planes 1352 / 1374, 104 planes 1382 / 1388 (the
+//             narrow transform), 108 planes 1473 / 1394; N = 128 66 planes
+//             172 / 216, 82 planes 282 / 234; N = 64 44 planes 86 / 86
 //   float64:  N = 256 122 planes 6887 / 8515; N = 128 82 planes 1057 / 1117,
 //             102 planes 1435 / 1231; N = 64 54 planes 214 / 229
 // (128 planes is also what the shared memory of the 8-byte types holds). Float32 and
